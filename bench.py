@@ -47,10 +47,11 @@ def bytes_per_node(model="bgk", storage="fp32", scalar="q7") -> int:
         return (q + ns) * 2 * 4
     return (q + ns) * 2 * 2 + (4 if scalar != "q6" else 0)
 PROFILE = os.path.join(ROOT, "profiles", "aa_step_bgk_fp32_traffic.md")
-# the sources that define the headline step kernel (bgk_step2_kernel)
+# the sources that define the headline step kernel (bgk_pair_kernel)
 KERNEL_SOURCES = ["paper_2112_08479_gb300/csrc/lbm_bgk.cu",
                   "paper_2112_08479_gb300/csrc/lbm_bgk_collide.cuh",
-                  "paper_2112_08479_gb300/csrc/lbm_aa2.cuh",
+                  "paper_2112_08479_gb300/csrc/lbm_lanes.cuh",
+                  "paper_2112_08479_gb300/csrc/lbm_pair.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_common.cuh"]
 
 
@@ -524,7 +525,7 @@ def run_ours(args, ws, rank, local):
     achieved = bpn * N / kern / 1e9
     headline = ((args.model, args.storage, args.scalar) == ("bgk", "fp32", "q7")
                 and args.workload == "config3")
-    kname = "bgk_step2_kernel" if args.model == "bgk" and WORKLOAD["nx"] % 2 == 0 else f"{args.model}_step_kernel"
+    kname = "bgk_pair_kernel" if args.model == "bgk" else "cumulant_step_kernel"
     if args.storage != "fp32" and args.scalar == "q7" and WORKLOAD["nx"] % 4 == 0:
         kname = f"{args.model}_even4_kernel + {kname}"
     traffic, tsrc = profiled_traffic(N) if headline else (None, "not captured for this variant")

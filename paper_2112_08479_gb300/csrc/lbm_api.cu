@@ -29,6 +29,7 @@ struct lbm_ctx {
     lbm_params p;
     KParams kp;
     Views v;
+    Sides sides;
     cudaStream_t stream;
     int64_t step;
     int odd;          // parity of the AA layout: the next step is odd when set
@@ -249,7 +250,9 @@ lbm_status lbm_init(const lbm_params* p, void* workspace, size_t bytes, void* cu
     c->v.devflags = (int*)(w + L.ddiag + sizeof(DevDiag));
     c->v.fgrad = (FrontGrad*)(w + L.fgrad);
     c->v.diag_blocks = L.nblocks;
+    c->v.sides = &c->sides;
     c->kp.devflags = c->v.devflags;
+    fill_sides(c->kp, kind(p), c->sides);
     cudaError_t e = launch_init(c->kp, kind(p), c->v, nullptr, p->x0, p->noise_amp,
                                 p->seed, c->stream);
     if (e != cudaSuccess) {
@@ -282,8 +285,7 @@ lbm_status lbm_step(lbm_ctx* c, int32_t nsteps) {
     if (!c) return arg_fail(nullptr, "ctx is NULL");
     if (nsteps < 0) return arg_fail(c, "nsteps must be >= 0");
     for (int32_t s = 0; s < nsteps; ++s) {
-        cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v.f, c->v.phi,
-                                    nullptr, c->stream);
+        cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, nullptr, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
         c->odd ^= 1;
         ++c->step;
@@ -296,8 +298,7 @@ lbm_status lbm_step_save(lbm_ctx* c, float* state_out) {
     if (!c) return arg_fail(nullptr, "ctx is NULL");
     if (!state_out) return arg_fail(c, "state_out is NULL");
     if (lbm_status s = narrow_check(c); s != LBM_OK) return s;
-    cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v.f, c->v.phi,
-                                state_out, c->stream);
+    cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, state_out, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
     c->odd ^= 1;
     ++c->step;
@@ -385,7 +386,7 @@ cudaError_t adjoint_step_any(lbm_ctx* c, const float* state, const float* lam_ne
 
 cudaError_t push_step_any(lbm_ctx* c, const float* src, float* dst, cudaStream_t st) {
     if (c->p.model == LBM_CUMULANT_Q27) return launch_cumulant_push_step(c->kp, src, dst, st);
-    return launch_push_step(c->kp, src, dst, st);
+    return launch_push_step(c->kp, c->sides, src, dst, st);
 }
 
 cudaStream_t stream_or_ctx(lbm_ctx* c, void* stream) {
@@ -437,8 +438,7 @@ lbm_status lbm_objective_forward(lbm_ctx* c, int32_t nsteps, int32_t K, float* c
             e = launch_get_state(c->kp, kind(&c->p), c->odd != 0, c->v,
                                  ckpt + (size_t)(n / K) * S, c->stream);
         if (e == cudaSuccess)
-            e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v.f, c->v.phi,
-                            nullptr, c->stream);
+            e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, nullptr, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "objective forward launch");
         c->odd ^= 1;
         ++c->step;

@@ -466,12 +466,17 @@ static cudaError_t dispatch(Kind k, Fn&& fn) {
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_step(const KParams& kp, Kind k, bool odd, void* f, void* phi, float* save,
+void fill_sides(const KParams& kp, Kind k, Sides& s) {
+    if (k.model == LBM_BGK_SMAG_Q19) fill_bgk_sides(kp, k.scalar, s);
+}
+
+cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, float* save,
                         cudaStream_t st) {
-    if (!save && staged_step_applies(kp, k)) return launch_staged_step(kp, k, odd, f, phi, st);
-    if (k.model == LBM_BGK_SMAG_Q19) return launch_bgk_step(kp, k.storage, k.scalar, odd, f, phi, save, st);
+    if (!save && staged_step_applies(kp, k)) return launch_staged_step(kp, k, odd, v.f, v.phi, st);
+    if (k.model == LBM_BGK_SMAG_Q19)
+        return launch_bgk_step(kp, k.storage, k.scalar, odd, v, save, st);
     if (k.model == LBM_CUMULANT_Q27)
-        return launch_cumulant_step(kp, k.storage, k.scalar, odd, f, phi, save, st);
+        return launch_cumulant_step(kp, k.storage, k.scalar, odd, v.f, v.phi, save, st);
     return cudaErrorInvalidValue;
 }
 

@@ -15,15 +15,24 @@
 //   Phi*_k = Phi_k - (Phi_k - w_k chi (1 + 4 c_k.u)) / tau_Phi     (Eq. 28-29)
 // followed by streaming (Eq. 17) in the AA pattern of lbm_common.cuh.
 //
-// The kernels are HBM-bound (about 2 flop per byte).  With nx even, one
-// thread owns two x-adjacent nodes and moves every population row as aligned
-// pairs (lbm_aa2.cuh): a warp reads and writes 256-byte row segments in FP32.
-// With nx odd, one thread per node.  No shared memory, no tensor cores.
+// FP32: two nodes per thread, x and x + 32 of a 64-node segment of a row
+// (lbm_pair.cuh), collided in packed arithmetic.  Large boxes are bound by HBM
+// (208 bytes per node update, about 2 flop per byte): 32.6 G node updates/s at
+// 2048x128x256, 1.00 of the measured copy rate, as the form before it (pairs
+// of adjacent nodes, collided one after the other).  Boxes that fit the L2 and
+// rows of odd length were bound by instruction issue: 322 instructions per
+// node on both parities (456 / 634 before on even / odd steps) take the step
+// from 17.4 to 12.8 us at 256x32x64 and from 35.3 to 28.8 us at 333x47x59.
+//
+// 16-bit storage: adjacent pairs (lbm_aa2.cuh) and, on even steps with nx a
+// multiple of 4, packed quads (lbm_quad.cuh); nx odd: one node per thread.
+// No shared memory, no tensor cores.
 #include <type_traits>
 
 #include "lbm_aa2.cuh"
 #include "lbm_bgk_collide.cuh"
 #include "lbm_internal.h"
+#include "lbm_pair.cuh"
 #include "lbm_quad.cuh"
 
 namespace lbmgpu {
@@ -51,12 +60,65 @@ __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_step_kernel(KParams kp
             save_pop(kp, save, 19 + NS, 19 + k, n,
                      s16 ? phi_canonical(kp, pv[k], ScalarLat<SL>::w(k)) : pv[k]);
     }
-    if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) collide_bgk<s16, SL>(kp, fv, pv);
+    if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
+        if constexpr (s16) collide_bgk<true, SL>(kp, fv, pv);
+        else collide_bgk_lanes<One, SL>(kp, kp.gx, kp.gy, kp.gz, fv, pv);
+    }
     if constexpr (R32) feed_rest<S>(pv);
     scatter<19, ODD, S, 0, false, true, Off>(kp, f, st, fv);
     scatter<NS, ODD, S, D0, R32, true, Off>(kp, phi, st, pv);
 }
 
+
+// FP32: two nodes per thread, x and x + 32 (lbm_pair.cuh), one code for both
+// parities, packed arithmetic.
+template <int SL, bool EDGE, bool SAVE, typename Off>
+__device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable<9, 3, Off>& tab,
+                                              float* __restrict__ f, float* __restrict__ phi,
+                                              float* __restrict__ save, bool odd, int x0, int y,
+                                              int z) {
+    constexpr int NS = ScalarLat<SL>::NS, D0 = ScalarLat<SL>::D0;
+    const PairNodes pn = pair_nodes(kp, x0, y, z, odd);
+    const int cls = pair_class(kp, odd, y, z);
+    const size_t fe = (size_t)19 * kp.N, pe = (size_t)NS * kp.N;
+    float2 fv[19], pv[NS];
+    pair_gather<9, 0, 19, float, EDGE>(kp, f, pn, tab.f[cls], fv);
+    pair_gather<3, D0, NS, float, EDGE>(kp, phi, pn, tab.g[cls], pv);
+    fv[0] = pair_ld_rest<float, EDGE>(kp, f, fe, pn);
+    if constexpr (SL == 7) pv[0] = pair_ld_rest<float, EDGE>(kp, phi, pe, pn);
+    if constexpr (SAVE) {
+        // on even steps the populations carry the names of their opposites
+        auto put = [&](int row, float2 v) {
+            if (pn.x < kp.nx) save_pop(kp, save, 19 + NS, row, pn.n, v.x);
+            if (pn.x + 32 < kp.nx) save_pop(kp, save, 19 + NS, row, pn.n + 32, v.y);
+        };
+#pragma unroll
+        for (int i = 0; i < 19; ++i) put(odd ? i : opp(i), fv[i]);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) put(19 + (odd ? k : opp(k + D0) - D0), pv[k]);
+    }
+    if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
+        const float s = odd ? 1.0f : -1.0f;   // even steps see the mirrored velocity set
+        collide_bgk_lanes<Two, SL>(kp, s * kp.gx, s * kp.gy, s * kp.gz, fv, pv);
+    }
+    pair_scatter<9, 0, 19, float, EDGE, false>(kp, f, pn, tab.f[cls], fv);
+    pair_scatter<3, D0, NS, float, EDGE, false>(kp, phi, pn, tab.g[cls], pv);
+    pair_st_rest<float, EDGE>(kp, f, fe, pn, fv[0]);
+    if constexpr (SL == 7) pair_st_rest<float, EDGE>(kp, phi, pe, pn, pv[0]);
+}
+
+template <int SL, bool SAVE, typename Off>
+__global__ void __launch_bounds__(128, LBM_PAIR_MINB)
+    bgk_pair_kernel(const __grid_constant__ KParams kp,
+                    const __grid_constant__ PairTable<9, 3, Off> tab, float* __restrict__ f,
+                    float* __restrict__ phi, float* __restrict__ save, bool odd) {
+    const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (x0 >= kp.nx) return;
+    if (pair_inner(kp, x0))
+        bgk_pair_step<SL, false, SAVE, Off>(kp, tab, f, phi, save, odd, x0, blockIdx.y, blockIdx.z);
+    else
+        bgk_pair_step<SL, true, SAVE, Off>(kp, tab, f, phi, save, odd, x0, blockIdx.y, blockIdx.z);
+}
 
 #ifndef LBM_BGK_ZSPLIT
 #define LBM_BGK_ZSPLIT 1
@@ -124,9 +186,6 @@ __global__ void __launch_bounds__(128, std::is_same<S, float>::value ? LBM_STEP2
     else bgk_step2_body<ODD, SAVE, S, SL, true, false, Off>(kp, f, phi, save, st);
 }
 
-#ifndef LBM_BGK_QUAD
-#define LBM_BGK_QUAD 1
-#endif
 #ifndef LBM_STEP4_MINB
 #define LBM_STEP4_MINB 3
 #endif
@@ -155,23 +214,44 @@ __global__ void __launch_bounds__(128, LBM_STEP4_MINB) bgk_even4_kernel(KParams 
 }
 
 template <typename S, int SL, typename Off>
-static cudaError_t launch_bgk_off(const KParams& kp, bool odd, S* f, S* phi, float* save,
-                                  cudaStream_t st) {
-    if constexpr (LBM_BGK_QUAD && !std::is_same<S, float>::value) {
-        if (!odd && !save && kp.nx % 4 == 0 && !(kp.flags & LBM_FLAG_ONE_NODE)) {
+static cudaError_t launch_bgk_off(const KParams& kp, const Sides& sides, bool odd, S* f, S* phi,
+                                  float* save, cudaStream_t st) {
+    // saved steps need (Q + NS) N < 2^32
+    constexpr bool narrow = std::is_same<Off, unsigned>::value;
+    if (save && !narrow) return cudaErrorInvalidValue;
+    if ((kp.flags & LBM_FLAG_ONE_NODE) || (!std::is_same<S, float>::value && kp.nx % 2)) {
+        dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
+        if (save) {
+            if (odd) bgk_step_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+            else bgk_step_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+        } else {
+            if (odd) bgk_step_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+            else bgk_step_kernel<false, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        }
+        return cudaGetLastError();
+    }
+    if constexpr (std::is_same<S, float>::value) {
+        const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
+        dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
+        const PairTable<9, 3, Off>& tab = pair_view<9, 3, Off>(sides);
+        if (save) {
+            if constexpr (narrow)
+                bgk_pair_kernel<SL, true, Off><<<grid, block, 0, st>>>(kp, tab, f, phi, save, odd);
+        } else {
+            bgk_pair_kernel<SL, false, Off><<<grid, block, 0, st>>>(kp, tab, f, phi, nullptr, odd);
+        }
+        return cudaGetLastError();
+    } else {
+        if (!odd && !save && kp.nx % 4 == 0) {
             dim3 block(128), grid((kp.nx / 4 + 127) / 128, kp.ny, kp.nz);
             bgk_even4_kernel<S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi);
             return cudaGetLastError();
         }
-    }
-    if constexpr (LBM_BGK_PAIR) if (kp.nx % 2 == 0 && !(kp.flags & LBM_FLAG_ONE_NODE)) {
         dim3 block(128), grid((kp.nx / 2 + 127) / 128, kp.ny, kp.nz);
         if (save) {
-            if constexpr (std::is_same<Off, unsigned>::value) {
+            if constexpr (narrow) {
                 if (odd) bgk_step2_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
                 else bgk_step2_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-            } else {
-                return cudaErrorInvalidValue;   // saved steps need (Q + NS) N < 2^32
             }
         } else {
             if (odd) bgk_step2_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
@@ -179,46 +259,38 @@ static cudaError_t launch_bgk_off(const KParams& kp, bool odd, S* f, S* phi, flo
         }
         return cudaGetLastError();
     }
-    dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-    if (save) {
-        if constexpr (std::is_same<Off, unsigned>::value) {
-            if (odd) bgk_step_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-            else bgk_step_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-        } else {
-            return cudaErrorInvalidValue;
-        }
-    } else {
-        if (odd) bgk_step_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-        else bgk_step_kernel<false, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-    }
-    return cudaGetLastError();
 }
 
-// 32-bit element offsets unless (Q + NS) N >= 2^32 (KParams::wide).
+void fill_bgk_sides(const KParams& kp, int scalar, Sides& s) {
+    const int d0 = scalar == LBM_SCALAR_Q6 ? 1 : 0;
+    // 32-bit element offsets unless (Q + NS) N >= 2^32 (KParams::wide)
+    if (kp.wide) pair_table(kp, d0, pair_view<9, 3, size_t>(s));
+    else pair_table(kp, d0, pair_view<9, 3, unsigned>(s));
+}
+
 template <typename S, int SL>
-static cudaError_t launch_bgk_typed(const KParams& kp, bool odd, S* f, S* phi, float* save,
-                                   cudaStream_t st) {
-    if (kp.wide) return launch_bgk_off<S, SL, size_t>(kp, odd, f, phi, save, st);
-    return launch_bgk_off<S, SL, unsigned>(kp, odd, f, phi, save, st);
+static cudaError_t launch_bgk_typed(const KParams& kp, bool odd, const Views& v, float* save,
+                                    cudaStream_t st) {
+    S *f = (S*)v.f, *phi = (S*)v.phi;
+    if (kp.wide) return launch_bgk_off<S, SL, size_t>(kp, *v.sides, odd, f, phi, save, st);
+    return launch_bgk_off<S, SL, unsigned>(kp, *v.sides, odd, f, phi, save, st);
 }
 
 template <int SL>
-static cudaError_t launch_bgk_sl(const KParams& kp, int storage, bool odd, void* f, void* phi,
+static cudaError_t launch_bgk_sl(const KParams& kp, int storage, bool odd, const Views& v,
                                  float* save, cudaStream_t st) {
     switch (storage) {
-        case LBM_FP32: return launch_bgk_typed<float, SL>(kp, odd, (float*)f, (float*)phi, save, st);
-        case LBM_FP16S: return launch_bgk_typed<__half, SL>(kp, odd, (__half*)f, (__half*)phi, save, st);
-        case LBM_BF16S:
-            return launch_bgk_typed<__nv_bfloat16, SL>(kp, odd, (__nv_bfloat16*)f,
-                                                       (__nv_bfloat16*)phi, save, st);
+        case LBM_FP32: return launch_bgk_typed<float, SL>(kp, odd, v, save, st);
+        case LBM_FP16S: return launch_bgk_typed<__half, SL>(kp, odd, v, save, st);
+        case LBM_BF16S: return launch_bgk_typed<__nv_bfloat16, SL>(kp, odd, v, save, st);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, void* f,
-                            void* phi, float* save, cudaStream_t st) {
-    if (scalar == LBM_SCALAR_Q7) return launch_bgk_sl<7>(kp, storage, odd, f, phi, save, st);
-    if (scalar == LBM_SCALAR_Q6) return launch_bgk_sl<6>(kp, storage, odd, f, phi, save, st);
+cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, const Views& v,
+                            float* save, cudaStream_t st) {
+    if (scalar == LBM_SCALAR_Q7) return launch_bgk_sl<7>(kp, storage, odd, v, save, st);
+    if (scalar == LBM_SCALAR_Q6) return launch_bgk_sl<6>(kp, storage, odd, v, save, st);
     return cudaErrorInvalidValue;
 }
 

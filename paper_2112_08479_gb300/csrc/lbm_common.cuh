@@ -158,12 +158,13 @@ __device__ __forceinline__ bool dbg_in(int* devflags, int flags, int site, const
 #ifndef LBM_STREAMING_HINTS
 #define LBM_STREAMING_HINTS 0
 #endif
-// Two nodes per thread with paired accesses when nx is even (lbm_aa2.cuh):
-// measured faster for the BGK model (all storages); the cumulant model, whose
-// collision needs more registers per node, keeps one node per thread.
-#ifndef LBM_BGK_PAIR
-#define LBM_BGK_PAIR 1
+// Resident blocks of the kernels with two nodes per thread (lbm_pair.cuh): 4 of
+// 128 threads, 128 registers.  5 (96 registers) spill 120 bytes and more and
+// measured slower.
+#ifndef LBM_PAIR_MINB
+#define LBM_PAIR_MINB 4
 #endif
+// Blocks of the 16-bit kernels with two adjacent nodes per thread (lbm_aa2.cuh).
 #ifndef LBM_STEP2_MINB
 #define LBM_STEP2_MINB 4
 #endif

@@ -23,6 +23,13 @@ struct FrontGrad {
     int valid;        // 1 when x + 1 < nx (the interpolated case)
 };
 
+// Where the two elements of each opposite pair of populations lie relative to
+// a node (lbm_pair.cuh), filled once per context: a host-side buffer that the
+// launchers pass to the kernels by value.
+struct Sides {
+    alignas(16) unsigned char bytes[3264];
+};
+
 // Workspace views handed to the launchers.
 struct Views {
     void* f;              // Q * N storage elements
@@ -36,11 +43,13 @@ struct Views {
     FrontGrad* fgrad;     // one record
     int* devflags;        // sticky device flags
     unsigned diag_blocks; // number of diagnostics blocks
+    const Sides* sides;   // host memory of the context
 };
 
 // Per-model step launchers (lbm_bgk.cu, lbm_cumulant.cu).
-cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, void* f,
-                            void* phi, float* save, cudaStream_t st);
+void fill_bgk_sides(const KParams& kp, int scalar, Sides& s);
+cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, const Views& v,
+                            float* save, cudaStream_t st);
 cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd, void* f,
                                  void* phi, float* save, cudaStream_t st);
 
@@ -56,8 +65,11 @@ bool staged_step_applies(const KParams& kp, Kind k);
 cudaError_t launch_staged_step(const KParams& kp, Kind k, bool odd, void* f, void* phi,
                                cudaStream_t st);
 
+// Fills a context's Sides for its box and kind.
+void fill_sides(const KParams& kp, Kind k, Sides& s);
+
 // odd: parity of the AA step.
-cudaError_t launch_step(const KParams& kp, Kind k, bool odd, void* f, void* phi, float* save,
+cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, float* save,
                         cudaStream_t st);
 cudaError_t launch_init(const KParams& kp, Kind k, const Views& v, const float* chi0, int x0,
                         double amp, uint64_t seed, cudaStream_t st);
@@ -73,7 +85,8 @@ cudaError_t launch_fw_accumulate(const KParams& kp, Kind k, bool odd, const View
                                  double* acc, double weight, cudaStream_t st);
 cudaError_t launch_adjoint_step(const KParams& kp, const float* state, const float* lam_next,
                                 float* lam, double* dcs, float wfw, float dAdCs, cudaStream_t st);
-cudaError_t launch_push_step(const KParams& kp, const float* src, float* dst, cudaStream_t st);
+cudaError_t launch_push_step(const KParams& kp, const Sides& sides, const float* src, float* dst,
+                             cudaStream_t st);
 cudaError_t launch_cumulant_adjoint_step(const KParams& kp, const float* state,
                                          const float* lam_next, float* lam, float wfw,
                                          cudaStream_t st);

@@ -47,9 +47,10 @@ def bytes_per_node(model="bgk", storage="fp32", scalar="q7") -> int:
         return (q + ns) * 2 * 4
     return (q + ns) * 2 * 2 + (4 if scalar != "q6" else 0)
 PROFILE = os.path.join(ROOT, "profiles", "aa_step_bgk_fp32_traffic.md")
-# the sources that define the headline step kernel (bgk_pair_kernel)
+# the sources that define the headline step kernel (bgk_chain_kernel)
 KERNEL_SOURCES = ["paper_2112_08479_gb300/csrc/lbm_bgk.cu",
                   "paper_2112_08479_gb300/csrc/lbm_bgk_collide.cuh",
+                  "paper_2112_08479_gb300/csrc/lbm_chain.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_lanes.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_pair.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_common.cuh"]
@@ -370,7 +371,9 @@ def timed_loop(lat, steps, warmup, torch, inner=INNER, with_diag=True, kernel_ev
     torch.cuda.synchronize()
     total = t0.elapsed_time(t1) / 1e3
     kern = sum(a.elapsed_time(b) for a, b in evs) / 1e3 / (steps * inner)
-    launches = steps * (inner + (2 if with_diag else 0))
+    # FP32 steps of one call share a launch (a whole box; slabs step one by one)
+    chained = getattr(lat, "peer", None) is None and lat.params.storage == 0
+    launches = steps * ((1 if chained else inner) + (2 if with_diag else 0))
     return total, kern, launches
 
 
@@ -525,7 +528,7 @@ def run_ours(args, ws, rank, local):
     achieved = bpn * N / kern / 1e9
     headline = ((args.model, args.storage, args.scalar) == ("bgk", "fp32", "q7")
                 and args.workload == "config3")
-    kname = "bgk_pair_kernel" if args.model == "bgk" else "cumulant_step_kernel"
+    kname = "bgk_chain_kernel" if args.model == "bgk" else "cumulant_step_kernel"
     if args.storage != "fp32" and args.scalar == "q7" and WORKLOAD["nx"] % 4 == 0:
         kname = f"{args.model}_even4_kernel + {kname}"
     traffic, tsrc = profiled_traffic(N) if headline else (None, "not captured for this variant")

@@ -119,10 +119,10 @@ typedef enum lbm_storage {
 /* sticky device flags reported in lbm_diagnostics.flags */
 #define LBM_DEVFLAG_NONFINITE 1   /* a macroscopic value was NaN or Inf */
 #define LBM_DEVFLAG_RHO_NONPOS 2  /* rho <= 0 at some node */
-#define LBM_DEVFLAG_TIMEOUT 4     /* a step kernel could not move its populations
-                                     through shared memory (a bounded wait for its
-                                     own bulk copies gave up, or the shared memory
-                                     was misaligned): the step is incomplete */
+#define LBM_DEVFLAG_TIMEOUT 4     /* a bounded wait of a step kernel gave up (for its
+                                     own bulk copies, or in a launch of several steps
+                                     for the step before), or its shared memory was
+                                     misaligned: the step is incomplete */
 #define LBM_DEVFLAG_BOUNDS 8      /* debug build: an index check failed and its access
                                      was skipped (lbm_debug_record) */
 
@@ -218,14 +218,17 @@ LBM_API lbm_status lbm_init(const lbm_params* p, void* workspace, size_t bytes,
  * lock field.  Resets the step counter. */
 LBM_API lbm_status lbm_set_scalar(lbm_ctx* ctx, const float* chi0);
 
-/* Advances nsteps >= 0 time steps (Eq. 17): one fused in-place kernel per
- * step (AA pattern: even steps collide in place, odd steps gather from and
- * scatter to the neighbours).  Asynchronous. */
+/* Advances nsteps >= 0 time steps (Eq. 17), each a fused in-place stream +
+ * collide pass (AA pattern: even steps collide in place, odd steps gather from
+ * and scatter to the neighbours); the steps of one call may share a launch.
+ * Asynchronous. */
 LBM_API lbm_status lbm_step(lbm_ctx* ctx, int32_t nsteps);
 
 /* One time step that also writes the pre-collision state of the current
  * step, in the canonical layout, to state_out ((Q + NS) * N floats, device).
- * Used to record the forward trajectory for the adjoint. */
+ * Used to record the forward trajectory for the adjoint: in FP32 it advances
+ * in the arithmetic of lbm_objective_forward and lbm_recompute_segment, which
+ * equals lbm_step's up to rounding. */
 LBM_API lbm_status lbm_step_save(lbm_ctx* ctx, float* state_out);
 
 /* Macroscopic fields of the current state (Eq. 19, 20 with the half-force
@@ -284,7 +287,7 @@ LBM_API lbm_status lbm_objective_forward(lbm_ctx* ctx, int32_t nsteps, int32_t K
  * scalar, FP32 storage):
  * from the checkpoint ckpt = s_{n0}, recomputes s_{n0+1} .. s_{n0+k-1} into
  * seg + j (Q + NS) N (j = 1 .. k-1; seg holds k states, slot 0 unused) with
- * an out-of-place step of the same arithmetic, then applies k adjoint steps
+ * an out-of-place step of lbm_objective_forward's arithmetic, then applies k adjoint steps
  * backwards: on entry lam holds lam_{n0+k}, on return lam_{n0}; the
  * friction of every state s_n with n >= 1 enters with weight w_fw (1 for the
  * time-integrated friction, 0 for an objective of the final state, e.g. the
@@ -299,8 +302,8 @@ LBM_API lbm_status lbm_adjoint_segment(lbm_ctx* ctx, const float* ckpt, int64_t 
  * recompute of one segment with the adjoint sweep of the next (two streams):
  *
  * lbm_recompute_segment: from ckpt = s_{n0}, writes s_{n0+1} .. s_{n0+k-1}
- * into seg + j (Q + NS) N, j = 1 .. k-1 (out-of-place steps of the same
- * arithmetic as lbm_step).
+ * into seg + j (Q + NS) N, j = 1 .. k-1 (out-of-place steps in the arithmetic
+ * of lbm_objective_forward, which equals lbm_step's up to FP32 rounding).
  *
  * lbm_adjoint_sweep: applies k adjoint steps backwards through ckpt (j = 0)
  * and seg + j (Q + NS) N (j = 1 .. k-1): on entry lam holds lam_{n0+k}, on

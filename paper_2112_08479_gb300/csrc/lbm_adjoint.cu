@@ -3,9 +3,9 @@
 // trajectory for it.  The objective is the time-integrated bottom friction
 // J = sum_n F_w(s_n) (Eq. 62-64); the step differentiated is Eq. 11, 17,
 // 19-30 and 32-35 as computed by collide_bgk.
+#include "lbm_aa2.cuh"
 #include "lbm_bgk_collide.cuh"
 #include "lbm_internal.h"
-#include "lbm_pair.cuh"
 
 namespace lbmgpu {
 
@@ -14,49 +14,77 @@ namespace lbmgpu {
 // recompute the forward trajectory inside the adjoint sweep: each node reads
 // its own populations at step n, collides, and pushes post-collision value i
 // to slot i of node x + c_i, or to slot opp(i) of itself across a wall
-// (Eq. 17).  Reading the own slots is the even AA step's gather (the mirrored
-// names of lbm_pair.cuh) and the push is the odd step's scatter, between two
-// arrays: the same arithmetic as the step kernels, 208 bytes per node, bound
-// by HBM.
-template <bool EDGE>
-__device__ __forceinline__ void bgk_push_body(const KParams& kp,
-                                              const PairTable<9, 3, unsigned>& tab,
-                                              const float* __restrict__ src,
-                                              float* __restrict__ dst, int x0, int y, int z) {
-    const size_t N = kp.N;
-    const float* sphi = src + 19 * N;
-    float* dphi = dst + 19 * N;
-    PairNodes pn = pair_nodes(kp, x0, y, z, false);
-    float2 f[19], p[7];
-    pair_gather<9, 0, 19, float, EDGE>(kp, src, pn, tab.f[0], f);
-    pair_gather<3, 0, 7, float, EDGE>(kp, sphi, pn, tab.g[0], p);
-    f[0] = pair_ld_rest<float, EDGE>(kp, src, 19 * N, pn);
-    p[0] = pair_ld_rest<float, EDGE>(kp, sphi, 7 * N, pn);
-    if (!(kp.flags & LBM_FLAG_NO_COLLIDE))
-        collide_bgk_lanes<Two, 7>(kp, -kp.gx, -kp.gy, -kp.gz, f, p);
-    pn.odd = true;
-    const int cls = pair_class(kp, true, y, z);
-    pair_scatter<9, 0, 19, float, EDGE, true>(kp, dst, pn, tab.f[cls], f);
-    pair_scatter<3, 0, 7, float, EDGE, true>(kp, dphi, pn, tab.g[cls], p);
-    pair_st_rest<float, EDGE>(kp, dst, 19 * N, pn, f[0]);
-    pair_st_rest<float, EDGE>(kp, dphi, 7 * N, pn, p[0]);
+// (Eq. 17).  Same arithmetic as the AA kernels, 208 bytes per node.
+__global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_push_kernel(KParams kp,
+                                                                      const float* __restrict__ src,
+                                                                      float* __restrict__ dst) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= kp.nx) return;
+    const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
+    const unsigned n = st.n, N = kp.N;
+    float f[19], p[7];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) f[i] = ld_chk(kp, LBM_SITE_ADJOINT, src, (unsigned)i * N + n, (size_t)26 * N);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) p[k] = ld_chk(kp, LBM_SITE_ADJOINT, src, (unsigned)(19 + k) * N + n, (size_t)26 * N);
+    if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) collide_bgk(kp, f, p);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        bool in = false;
+        const unsigned d = i == 0 ? n : nbr(st, cx27(i), cy27(i), cz27(i), in);
+        st_chk(kp, LBM_SITE_ADJOINT, dst, (i != 0 && in) ? (unsigned)i * N + d : (unsigned)opp(i) * N + n,
+               (size_t)26 * N, f[i]);
+    }
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        bool in = false;
+        const unsigned d = k == 0 ? n : nbr(st, cx27(k), cy27(k), cz27(k), in);
+        st_chk(kp, LBM_SITE_ADJOINT, dst,
+               (k != 0 && in) ? (unsigned)(19 + k) * N + d : (unsigned)(19 + opp(k)) * N + n,
+               (size_t)26 * N, p[k]);
+    }
 }
 
-__global__ void __launch_bounds__(128, LBM_PAIR_MINB)
-    bgk_push_kernel(const __grid_constant__ KParams kp,
-                    const __grid_constant__ PairTable<9, 3, unsigned> tab,
-                    const float* __restrict__ src, float* __restrict__ dst) {
-    const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
-    if (x0 >= kp.nx) return;
-    if (pair_inner(kp, x0)) bgk_push_body<false>(kp, tab, src, dst, x0, blockIdx.y, blockIdx.z);
-    else bgk_push_body<true>(kp, tab, src, dst, x0, blockIdx.y, blockIdx.z);
+// The same push for two x-adjacent nodes per thread (nx even): reading the
+// own slots is the AA even-step gather and pushing to slot i of node x + c_i
+// (own slot opp(i) across a wall) is the AA odd-step scatter, both with
+// paired accesses (lbm_aa2.cuh), here between two arrays.
+template <bool ZW>
+__device__ __forceinline__ void bgk_push2_body(const KParams& kp, const float* __restrict__ src,
+                                               float* __restrict__ dst, const Stencil2& st) {
+    const unsigned N = kp.N;
+    float f0[19], f1[19], p0[7], p1[7];
+    gather2<19, false>(kp, src, st, f0, f1);
+    gather2<7, false>(kp, src + (size_t)19 * N, st, p0, p1);
+    if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
+        collide_bgk(kp, f0, p0);
+        collide_bgk(kp, f1, p1);
+    }
+    scatter2<19, true, float, 0, false, ZW>(kp, dst, st, f0, f1);
+    scatter2<7, true, float, 0, false, ZW>(kp, dst + (size_t)19 * N, st, p0, p1);
 }
 
-cudaError_t launch_push_step(const KParams& kp, const Sides& sides, const float* src, float* dst,
-                             cudaStream_t st) {
-    const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
-    dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
-    bgk_push_kernel<<<grid, block, 0, st>>>(kp, pair_view<9, 3, unsigned>(sides), src, dst);
+__global__ void __launch_bounds__(128, LBM_STEP2_MINB) bgk_push2_kernel(KParams kp,
+                                                                      const float* __restrict__ src,
+                                                                      float* __restrict__ dst) {
+    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const Stencil2 st = make_stencil2(kp, x, blockIdx.y, blockIdx.z);
+    const int z = blockIdx.z;
+    // rows away from the z walls (uniform per block) skip the wall selects
+    if ((kp.flags & LBM_FLAG_PERIODIC_Z) || (z > 0 && z < kp.nz - 1))
+        bgk_push2_body<false>(kp, src, dst, st);
+    else
+        bgk_push2_body<true>(kp, src, dst, st);
+}
+
+cudaError_t launch_push_step(const KParams& kp, const float* src, float* dst, cudaStream_t st) {
+    if (kp.nx % 2 == 0) {
+        dim3 block(128), grid((kp.nx / 2 + 127) / 128, kp.ny, kp.nz);
+        bgk_push2_kernel<<<grid, block, 0, st>>>(kp, src, dst);
+        return cudaGetLastError();
+    }
+    dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
+    bgk_push_kernel<<<grid, block, 0, st>>>(kp, src, dst);
     return cudaGetLastError();
 }
 

@@ -284,12 +284,10 @@ lbm_status lbm_step(lbm_ctx* c, int32_t nsteps) {
     const Range range("lbm_step");
     if (!c) return arg_fail(nullptr, "ctx is NULL");
     if (nsteps < 0) return arg_fail(c, "nsteps must be >= 0");
-    for (int32_t s = 0; s < nsteps; ++s) {
-        cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, nullptr, c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
-        c->odd ^= 1;
-        ++c->step;
-    }
+    const cudaError_t e = launch_steps(c->kp, kind(&c->p), c->odd != 0, nsteps, c->v, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+    c->odd ^= nsteps & 1;
+    c->step += nsteps;
     return LBM_OK;
 }
 
@@ -298,7 +296,7 @@ lbm_status lbm_step_save(lbm_ctx* c, float* state_out) {
     if (!c) return arg_fail(nullptr, "ctx is NULL");
     if (!state_out) return arg_fail(c, "state_out is NULL");
     if (lbm_status s = narrow_check(c); s != LBM_OK) return s;
-    cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, state_out, c->stream);
+    cudaError_t e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, state_out, true, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
     c->odd ^= 1;
     ++c->step;
@@ -386,7 +384,7 @@ cudaError_t adjoint_step_any(lbm_ctx* c, const float* state, const float* lam_ne
 
 cudaError_t push_step_any(lbm_ctx* c, const float* src, float* dst, cudaStream_t st) {
     if (c->p.model == LBM_CUMULANT_Q27) return launch_cumulant_push_step(c->kp, src, dst, st);
-    return launch_push_step(c->kp, c->sides, src, dst, st);
+    return launch_push_step(c->kp, src, dst, st);
 }
 
 cudaStream_t stream_or_ctx(lbm_ctx* c, void* stream) {
@@ -438,7 +436,7 @@ lbm_status lbm_objective_forward(lbm_ctx* c, int32_t nsteps, int32_t K, float* c
             e = launch_get_state(c->kp, kind(&c->p), c->odd != 0, c->v,
                                  ckpt + (size_t)(n / K) * S, c->stream);
         if (e == cudaSuccess)
-            e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, nullptr, c->stream);
+            e = launch_step(c->kp, kind(&c->p), c->odd != 0, c->v, nullptr, true, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "objective forward launch");
         c->odd ^= 1;
         ++c->step;

@@ -14,6 +14,7 @@
 // has a fixed order, so results are bitwise reproducible.
 #include <type_traits>
 
+#include "lbm_chain.cuh"
 #include "lbm_internal.h"
 
 namespace lbmgpu {
@@ -347,6 +348,82 @@ __global__ void adjoint_chi0_kernel(unsigned N, int Q, const float* __restrict__
     grad[n] = g;
 }
 
+// Rules of the chain (lbm_chain.cuh).
+cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, unsigned unit_nodes,
+                       unsigned warps, int nsteps, bool odd, ChainPlan& out, bool& ran) {
+    // A box whose state stays in L2 needs no wave: steps in turn, one slot.
+    constexpr double RESIDENT = 70e6;
+    // Otherwise four slots where the planes between the first and the last one
+    // stay in L2 (64 MB: the L2 still serves a working set of that size at its
+    // full rate), else three, on slabs along x as narrow as that takes.  FP32 BGK,
+    // G node updates/s with 1 step per launch and 2, 3, 4, 6 slots: 512x64x64 30.7,
+    // 44.8, 46.8, 47.4, 46.1; 1024x64x128 32.9, 43.7, 45.6, 45.8, 38.5; 2500x150x100
+    // with periodic ends 32.7, 32.6, 35.9, 35.7, 31.3; 2048x128x256 32.8, 35.5,
+    // 39.5, 39.5, 36.8 (three slots in 1, 2, 3 slabs: 34.7, 36.2, 39.5).
+    constexpr int SLOTS = 4, SLOTS_SLABS = 3;
+    constexpr double LIVE = 64e6;
+    // Distance of the slots beyond the plane they need, in items in flight
+    // (2.5 per computing warp group: published, polled and drawn items): 1.5,
+    // 2, 2.5, 3 measured 262, 210, 199, 198 us at 1024x64x128.
+    constexpr double SLACK = 2.5;
+    ran = false;
+    ChainParams& p = out.p;
+    const bool resident = plane_bytes * (double)kp.nz <= RESIDENT;
+    // a single step gains nothing, a few steps of a small box not the reset of
+    // the counters (about two launches' worth)
+    if (nsteps < (resident ? 4 : 2)) return cudaSuccess;
+    if (!resident && (kp.flags & LBM_FLAG_PERIODIC_Z)) return cudaSuccess;   // a wave needs an end
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const unsigned nx = (unsigned)kp.nx, ny = (unsigned)kp.ny, nz = (unsigned)kp.nz;
+    p.sync = reinterpret_cast<unsigned*>(v.stage);
+    p.nsteps = nsteps;
+    p.odd0 = odd ? 1 : 0;
+    p.ns = (nx + unit_nodes - 1) / unit_nodes;
+    // units per item: as many as keep the feeding warp ahead of the others, but
+    // no fewer items than there are warps to share them (128x8x16: 3.9 us per
+    // step with 1, 4.4 with 2, 5.1 with 4; 256x32x16: 8.6, 4.8, 5.1)
+    const double units = (double)p.ns * ny * nz;
+    p.U = units < 0.5 * sms * warps ? 1 : (units < 2.0 * sms * warps ? 2 : 4);
+    int T = resident ? 1 : (nsteps < SLOTS ? nsteps : SLOTS);
+    unsigned M, bpt, P, sw, nslab;
+    for (;; --T) {
+        double live = 0.0;
+        for (nslab = 1;; ++nslab) {
+            p.skew = nslab == 1 ? 0 : ((kp.flags & LBM_FLAG_PERIODIC_X) ? 2 : 1);
+            sw = (p.ns + p.skew * (unsigned)(T - 1) + nslab - 1) / nslab;
+            for (p.R = 1; (sw * p.R) % p.U && p.R < p.U && p.R < ny;) p.R *= 2;
+            M = (ny + p.R - 1) / p.R;
+            bpt = (sw * p.R + p.U - 1) / p.U;
+            P = M * nz;
+            p.lag = T == 1 ? 0 : M + 3 + (unsigned)(SLACK * sms * warps / p.U / (T * bpt));
+            live = ((double)(T - 1) * p.lag / M + 1.0) * plane_bytes * sw / p.ns;
+            if (T == 1 || live <= LIVE || sw <= 8 || T > SLOTS_SLABS) break;
+        }
+        if (T > SLOTS_SLABS && live > LIVE) continue;
+        if (T == 1 || (double)(T - 1) * p.lag + 2.0 * M <= P) break;
+    }
+    if (T == 1 && !resident) return cudaSuccess;   // too few planes for a wave
+    if (CHAIN_COUNTERS + (size_t)P > kp.N) return cudaSuccess;
+    p.T = T;
+    p.groups = (unsigned)((nsteps + T - 1) / T) * nslab;
+    const double total = ((double)p.groups * P + (double)(T - 1) * p.lag) * T * bpt;
+    if (total >= 2147000000.0) return cudaSuccess;   // 31-bit tickets
+    p.total = (unsigned)total;
+    p.M.set(M);
+    p.bpt.set(bpt);
+    p.per.set((unsigned)T * bpt);
+    p.P.set(P);
+    p.nslab.set(nslab);
+    p.sw.set(sw);
+    p.Ud.set(p.U);
+    out.grid = (unsigned)sms < p.total ? (unsigned)sms : p.total;
+    ran = true;
+    return cudaSuccess;
+}
+
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
@@ -471,13 +548,27 @@ void fill_sides(const KParams& kp, Kind k, Sides& s) {
 }
 
 cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, float* save,
-                        cudaStream_t st) {
+                        bool trajectory, cudaStream_t st) {
     if (!save && staged_step_applies(kp, k)) return launch_staged_step(kp, k, odd, v.f, v.phi, st);
     if (k.model == LBM_BGK_SMAG_Q19)
-        return launch_bgk_step(kp, k.storage, k.scalar, odd, v, save, st);
+        return launch_bgk_step(kp, k.storage, k.scalar, odd, v, save, trajectory, st);
     if (k.model == LBM_CUMULANT_Q27)
         return launch_cumulant_step(kp, k.storage, k.scalar, odd, v.f, v.phi, save, st);
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
+                         cudaStream_t st) {
+    bool ran = false;
+    if (nsteps >= 2 && k.model == LBM_BGK_SMAG_Q19) {
+        const cudaError_t e = launch_bgk_chain(kp, k.storage, k.scalar, odd, nsteps, v, ran, st);
+        if (e != cudaSuccess || ran) return e;
+    }
+    for (int s = 0; s < nsteps; ++s) {
+        const cudaError_t e = launch_step(kp, k, odd != ((s & 1) != 0), v, nullptr, false, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_init(const KParams& kp, Kind k, const Views& v, const float* chi0, int x0,

@@ -31,13 +31,16 @@
 
 #include "lbm_aa2.cuh"
 #include "lbm_bgk_collide.cuh"
+#include "lbm_chain.cuh"
 #include "lbm_internal.h"
 #include "lbm_pair.cuh"
 #include "lbm_quad.cuh"
 
 namespace lbmgpu {
 
-template <bool ODD, bool SAVE, typename S, int SL, typename Off = unsigned>
+// CONTRACT: FP32 in the compiler-contracted arithmetic (collide_bgk), as the
+// 16-bit forms always.
+template <bool ODD, bool SAVE, typename S, int SL, typename Off = unsigned, bool CONTRACT = false>
 __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_step_kernel(KParams kp, S* __restrict__ f,
                                                        S* __restrict__ phi,
                                                        float* __restrict__ save) {
@@ -61,7 +64,7 @@ __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_step_kernel(KParams kp
                      s16 ? phi_canonical(kp, pv[k], ScalarLat<SL>::w(k)) : pv[k]);
     }
     if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
-        if constexpr (s16) collide_bgk<true, SL>(kp, fv, pv);
+        if constexpr (s16 || CONTRACT) collide_bgk<s16, SL>(kp, fv, pv);
         else collide_bgk_lanes<One, SL>(kp, kp.gx, kp.gy, kp.gz, fv, pv);
     }
     if constexpr (R32) feed_rest<S>(pv);
@@ -72,11 +75,10 @@ __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_step_kernel(KParams kp
 
 // FP32: two nodes per thread, x and x + 32 (lbm_pair.cuh), one code for both
 // parities, packed arithmetic.
-template <int SL, bool EDGE, bool SAVE, typename Off>
+template <int SL, bool EDGE, typename Off>
 __device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable<9, 3, Off>& tab,
                                               float* __restrict__ f, float* __restrict__ phi,
-                                              float* __restrict__ save, bool odd, int x0, int y,
-                                              int z) {
+                                              bool odd, int x0, int y, int z) {
     constexpr int NS = ScalarLat<SL>::NS, D0 = ScalarLat<SL>::D0;
     const PairNodes pn = pair_nodes(kp, x0, y, z, odd);
     const int cls = pair_class(kp, odd, y, z);
@@ -86,17 +88,6 @@ __device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable
     pair_gather<3, D0, NS, float, EDGE>(kp, phi, pn, tab.g[cls], pv);
     fv[0] = pair_ld_rest<float, EDGE>(kp, f, fe, pn);
     if constexpr (SL == 7) pv[0] = pair_ld_rest<float, EDGE>(kp, phi, pe, pn);
-    if constexpr (SAVE) {
-        // on even steps the populations carry the names of their opposites
-        auto put = [&](int row, float2 v) {
-            if (pn.x < kp.nx) save_pop(kp, save, 19 + NS, row, pn.n, v.x);
-            if (pn.x + 32 < kp.nx) save_pop(kp, save, 19 + NS, row, pn.n + 32, v.y);
-        };
-#pragma unroll
-        for (int i = 0; i < 19; ++i) put(odd ? i : opp(i), fv[i]);
-#pragma unroll
-        for (int k = 0; k < NS; ++k) put(19 + (odd ? k : opp(k + D0) - D0), pv[k]);
-    }
     if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
         const float s = odd ? 1.0f : -1.0f;   // even steps see the mirrored velocity set
         collide_bgk_lanes<Two, SL>(kp, s * kp.gx, s * kp.gy, s * kp.gz, fv, pv);
@@ -107,17 +98,17 @@ __device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable
     if constexpr (SL == 7) pair_st_rest<float, EDGE>(kp, phi, pe, pn, pv[0]);
 }
 
-template <int SL, bool SAVE, typename Off>
+template <int SL, typename Off>
 __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
     bgk_pair_kernel(const __grid_constant__ KParams kp,
                     const __grid_constant__ PairTable<9, 3, Off> tab, float* __restrict__ f,
-                    float* __restrict__ phi, float* __restrict__ save, bool odd) {
+                    float* __restrict__ phi, bool odd) {
     const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (x0 >= kp.nx) return;
     if (pair_inner(kp, x0))
-        bgk_pair_step<SL, false, SAVE, Off>(kp, tab, f, phi, save, odd, x0, blockIdx.y, blockIdx.z);
+        bgk_pair_step<SL, false, Off>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
     else
-        bgk_pair_step<SL, true, SAVE, Off>(kp, tab, f, phi, save, odd, x0, blockIdx.y, blockIdx.z);
+        bgk_pair_step<SL, true, Off>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
 }
 
 #ifndef LBM_BGK_ZSPLIT
@@ -213,52 +204,106 @@ __global__ void __launch_bounds__(128, LBM_STEP4_MINB) bgk_even4_kernel(KParams 
     even4_body<19, SL, S, Off, BgkQuadCollide>(kp, f, phi);
 }
 
+// Many steps in one launch (lbm_chain.cuh).  14 computing warps: 128 registers
+// without spills (18 warps at 96 registers spill 244 bytes and measured 28
+// against 39 G node updates/s at 2048x128x256).  The body has to be small: with
+// the former step kernels inlined (four bodies of 17 to 20 KB) the mixed
+// parities missed the instruction cache (3.3 of 11.6 cycles per issue) and ran
+// at 26 G.  Per step, one launch each -> chain: 128x8x16 4.4 -> 3.9 us,
+// 256x32x64 12.8 -> 10.1, 333x47x59 28.8 -> 23.3, 1024x64x128 256 -> 183,
+// 2048x128x256 2050 -> 1690 (39.6 G node updates/s, 8.2 TB/s of populations).
+constexpr int BGK_CHAIN_WARPS = 14;
+template <int SL>
+__global__ void __launch_bounds__(32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 1)
+    bgk_chain_kernel(const __grid_constant__ KParams kp, const __grid_constant__ ChainParams cp,
+                     const __grid_constant__ PairTable<9, 3, unsigned> tab, float* __restrict__ f,
+                     float* __restrict__ phi) {
+    chain_run<BGK_CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
+        const int x0 = 64 * seg;
+        if (pair_inner(kp, x0))
+            bgk_pair_step<SL, false, unsigned>(kp, tab, f, phi, odd, x0, y, z);
+        else
+            bgk_pair_step<SL, true, unsigned>(kp, tab, f, phi, odd, x0, y, z);
+    });
+}
+
+template <int SL>
+static cudaError_t chain_typed(const KParams& kp, bool odd, int nsteps, const Views& v, bool& ran,
+                               cudaStream_t st) {
+    ChainPlan pl;
+    cudaError_t e = chain_plan(kp, v, (size_t)kp.nxny * (19 + ScalarLat<SL>::NS) * sizeof(float), 64,
+                               BGK_CHAIN_WARPS, nsteps, odd, pl, ran);
+    if (e != cudaSuccess || !ran) return e;
+    e = cudaMemsetAsync(pl.p.sync, 0, chain_sync_bytes(pl.p), st);
+    if (e != cudaSuccess) return e;
+    bgk_chain_kernel<SL><<<pl.grid, 32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 0, st>>>(
+        kp, pl.p, pair_view<9, 3, unsigned>(*v.sides), (float*)v.f, (float*)v.phi);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bgk_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
+                             const Views& v, bool& ran, cudaStream_t st) {
+    ran = false;
+    if (storage != LBM_FP32 || kp.wide || (kp.flags & LBM_FLAG_ONE_NODE)) return cudaSuccess;
+    return scalar == LBM_SCALAR_Q7 ? chain_typed<7>(kp, odd, nsteps, v, ran, st)
+                                   : chain_typed<6>(kp, odd, nsteps, v, ran, st);
+}
+
+// The steps in the contracted arithmetic: every 16-bit step, and in FP32 the
+// saved steps, the trajectory of an objective (lbm_objective_forward) and, in
+// lbm_adjoint.cu, its recompute in the reverse sweep, which have to retrace each
+// other.  (A gradient of the front divides by differences of chi of a few 1e-3
+// at chi ~ 0.02, held as chi - 1 in FP32: its error, 1e-6 to 3e-5, is the
+// rounding of this one trajectory, so another arithmetic, however accurate,
+// gives another error of the same size; these paths keep theirs.)
 template <typename S, int SL, typename Off>
-static cudaError_t launch_bgk_off(const KParams& kp, const Sides& sides, bool odd, S* f, S* phi,
-                                  float* save, cudaStream_t st) {
+static cudaError_t launch_bgk_contracted(const KParams& kp, bool odd, S* f, S* phi, float* save,
+                                         cudaStream_t st) {
     // saved steps need (Q + NS) N < 2^32
     constexpr bool narrow = std::is_same<Off, unsigned>::value;
     if (save && !narrow) return cudaErrorInvalidValue;
-    if ((kp.flags & LBM_FLAG_ONE_NODE) || (!std::is_same<S, float>::value && kp.nx % 2)) {
+    if ((kp.flags & LBM_FLAG_ONE_NODE) || kp.nx % 2) {
         dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
         if (save) {
-            if (odd) bgk_step_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-            else bgk_step_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+            if (odd) bgk_step_kernel<true, true, S, SL, unsigned, true><<<grid, block, 0, st>>>(kp, f, phi, save);
+            else bgk_step_kernel<false, true, S, SL, unsigned, true><<<grid, block, 0, st>>>(kp, f, phi, save);
         } else {
-            if (odd) bgk_step_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-            else bgk_step_kernel<false, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+            if (odd) bgk_step_kernel<true, false, S, SL, Off, true><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+            else bgk_step_kernel<false, false, S, SL, Off, true><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
         }
         return cudaGetLastError();
     }
-    if constexpr (std::is_same<S, float>::value) {
-        const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
-        dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
-        const PairTable<9, 3, Off>& tab = pair_view<9, 3, Off>(sides);
-        if (save) {
-            if constexpr (narrow)
-                bgk_pair_kernel<SL, true, Off><<<grid, block, 0, st>>>(kp, tab, f, phi, save, odd);
-        } else {
-            bgk_pair_kernel<SL, false, Off><<<grid, block, 0, st>>>(kp, tab, f, phi, nullptr, odd);
-        }
-        return cudaGetLastError();
-    } else {
+    if constexpr (!std::is_same<S, float>::value) {
         if (!odd && !save && kp.nx % 4 == 0) {
             dim3 block(128), grid((kp.nx / 4 + 127) / 128, kp.ny, kp.nz);
             bgk_even4_kernel<S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi);
             return cudaGetLastError();
         }
-        dim3 block(128), grid((kp.nx / 2 + 127) / 128, kp.ny, kp.nz);
-        if (save) {
-            if constexpr (narrow) {
-                if (odd) bgk_step2_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-                else bgk_step2_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-            }
-        } else {
-            if (odd) bgk_step2_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-            else bgk_step2_kernel<false, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-        }
+    }
+    dim3 block(128), grid((kp.nx / 2 + 127) / 128, kp.ny, kp.nz);
+    if (save) {
+        if (odd) bgk_step2_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+        else bgk_step2_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+    } else {
+        if (odd) bgk_step2_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        else bgk_step2_kernel<false, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+    }
+    return cudaGetLastError();
+}
+
+template <int SL, typename Off>
+static cudaError_t launch_bgk_fp32(const KParams& kp, const Sides& sides, bool odd, float* f,
+                                   float* phi, cudaStream_t st) {
+    if (kp.flags & LBM_FLAG_ONE_NODE) {
+        dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
+        if (odd) bgk_step_kernel<true, false, float, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        else bgk_step_kernel<false, false, float, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
         return cudaGetLastError();
     }
+    const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
+    dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
+    bgk_pair_kernel<SL, Off><<<grid, block, 0, st>>>(kp, pair_view<9, 3, Off>(sides), f, phi, odd);
+    return cudaGetLastError();
 }
 
 void fill_bgk_sides(const KParams& kp, int scalar, Sides& s) {
@@ -270,27 +315,32 @@ void fill_bgk_sides(const KParams& kp, int scalar, Sides& s) {
 
 template <typename S, int SL>
 static cudaError_t launch_bgk_typed(const KParams& kp, bool odd, const Views& v, float* save,
-                                    cudaStream_t st) {
+                                    bool trajectory, cudaStream_t st) {
     S *f = (S*)v.f, *phi = (S*)v.phi;
-    if (kp.wide) return launch_bgk_off<S, SL, size_t>(kp, *v.sides, odd, f, phi, save, st);
-    return launch_bgk_off<S, SL, unsigned>(kp, *v.sides, odd, f, phi, save, st);
+    if constexpr (std::is_same<S, float>::value) {
+        if (!save && !trajectory)
+            return kp.wide ? launch_bgk_fp32<SL, size_t>(kp, *v.sides, odd, f, phi, st)
+                           : launch_bgk_fp32<SL, unsigned>(kp, *v.sides, odd, f, phi, st);
+    }
+    return kp.wide ? launch_bgk_contracted<S, SL, size_t>(kp, odd, f, phi, save, st)
+                   : launch_bgk_contracted<S, SL, unsigned>(kp, odd, f, phi, save, st);
 }
 
 template <int SL>
 static cudaError_t launch_bgk_sl(const KParams& kp, int storage, bool odd, const Views& v,
-                                 float* save, cudaStream_t st) {
+                                 float* save, bool trajectory, cudaStream_t st) {
     switch (storage) {
-        case LBM_FP32: return launch_bgk_typed<float, SL>(kp, odd, v, save, st);
-        case LBM_FP16S: return launch_bgk_typed<__half, SL>(kp, odd, v, save, st);
-        case LBM_BF16S: return launch_bgk_typed<__nv_bfloat16, SL>(kp, odd, v, save, st);
+        case LBM_FP32: return launch_bgk_typed<float, SL>(kp, odd, v, save, trajectory, st);
+        case LBM_FP16S: return launch_bgk_typed<__half, SL>(kp, odd, v, save, trajectory, st);
+        case LBM_BF16S: return launch_bgk_typed<__nv_bfloat16, SL>(kp, odd, v, save, trajectory, st);
     }
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, const Views& v,
-                            float* save, cudaStream_t st) {
-    if (scalar == LBM_SCALAR_Q7) return launch_bgk_sl<7>(kp, storage, odd, v, save, st);
-    if (scalar == LBM_SCALAR_Q6) return launch_bgk_sl<6>(kp, storage, odd, v, save, st);
+                            float* save, bool trajectory, cudaStream_t st) {
+    if (scalar == LBM_SCALAR_Q7) return launch_bgk_sl<7>(kp, storage, odd, v, save, trajectory, st);
+    if (scalar == LBM_SCALAR_Q6) return launch_bgk_sl<6>(kp, storage, odd, v, save, trajectory, st);
     return cudaErrorInvalidValue;
 }
 

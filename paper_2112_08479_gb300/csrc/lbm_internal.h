@@ -49,7 +49,9 @@ struct Views {
 // Per-model step launchers (lbm_bgk.cu, lbm_cumulant.cu).
 void fill_bgk_sides(const KParams& kp, int scalar, Sides& s);
 cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, const Views& v,
-                            float* save, cudaStream_t st);
+                            float* save, bool trajectory, cudaStream_t st);
+cudaError_t launch_bgk_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
+                             const Views& v, bool& ran, cudaStream_t st);
 cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd, void* f,
                                  void* phi, float* save, cudaStream_t st);
 
@@ -68,9 +70,13 @@ cudaError_t launch_staged_step(const KParams& kp, Kind k, bool odd, void* f, voi
 // Fills a context's Sides for its box and kind.
 void fill_sides(const KParams& kp, Kind k, Sides& s);
 
-// odd: parity of the AA step.
+// odd: parity of the AA step.  trajectory: a step that the adjoint retraces
+// (lbm_objective_forward; saved steps always are).
 cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, float* save,
-                        cudaStream_t st);
+                        bool trajectory, cudaStream_t st);
+// nsteps steps, the first of parity `odd`.
+cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
+                         cudaStream_t st);
 cudaError_t launch_init(const KParams& kp, Kind k, const Views& v, const float* chi0, int x0,
                         double amp, uint64_t seed, cudaStream_t st);
 cudaError_t launch_macros(const KParams& kp, Kind k, bool odd, const Views& v, float* rho,
@@ -85,8 +91,7 @@ cudaError_t launch_fw_accumulate(const KParams& kp, Kind k, bool odd, const View
                                  double* acc, double weight, cudaStream_t st);
 cudaError_t launch_adjoint_step(const KParams& kp, const float* state, const float* lam_next,
                                 float* lam, double* dcs, float wfw, float dAdCs, cudaStream_t st);
-cudaError_t launch_push_step(const KParams& kp, const Sides& sides, const float* src, float* dst,
-                             cudaStream_t st);
+cudaError_t launch_push_step(const KParams& kp, const float* src, float* dst, cudaStream_t st);
 cudaError_t launch_cumulant_adjoint_step(const KParams& kp, const float* state,
                                          const float* lam_next, float* lam, float wfw,
                                          cudaStream_t st);

@@ -371,8 +371,10 @@ def timed_loop(lat, steps, warmup, torch, inner=INNER, with_diag=True, kernel_ev
     torch.cuda.synchronize()
     total = t0.elapsed_time(t1) / 1e3
     kern = sum(a.elapsed_time(b) for a, b in evs) / 1e3 / (steps * inner)
-    # FP32 steps of one call share a launch (a whole box; slabs step one by one)
-    chained = getattr(lat, "peer", None) is None and lat.params.storage == 0
+    # FP32 steps of one call share a launch (a whole box; slabs step one by one),
+    # except with the D3Q27 scalar
+    chained = (getattr(lat, "peer", None) is None and lat.params.storage == 0
+               and lat.params.scalar != 2)
     launches = steps * ((1 if chained else inner) + (2 if with_diag else 0))
     return total, kern, launches
 
@@ -528,9 +530,12 @@ def run_ours(args, ws, rank, local):
     achieved = bpn * N / kern / 1e9
     headline = ((args.model, args.storage, args.scalar) == ("bgk", "fp32", "q7")
                 and args.workload == "config3")
-    kname = "bgk_chain_kernel" if args.model == "bgk" else "cumulant_step_kernel"
-    if args.storage != "fp32" and args.scalar == "q7" and WORKLOAD["nx"] % 4 == 0:
-        kname = f"{args.model}_even4_kernel + {kname}"
+    if args.storage == "fp32":
+        kname = "cumulant_step_kernel" if args.scalar == "q27" else f"{args.model}_chain_kernel"
+    else:
+        kname = "bgk_step2_kernel" if args.model == "bgk" else "cumulant_step_kernel"
+        if args.scalar == "q7" and WORKLOAD["nx"] % 4 == 0:
+            kname = f"{args.model}_even4_kernel + {kname}"
     traffic, tsrc = profiled_traffic(N) if headline else (None, "not captured for this variant")
     roof = {"bound": "hbm",
             "kernel": f"{kname} (AA even/odd, {args.storage.upper()})",

@@ -545,6 +545,7 @@ static cudaError_t dispatch(Kind k, Fn&& fn) {
 
 void fill_sides(const KParams& kp, Kind k, Sides& s) {
     if (k.model == LBM_BGK_SMAG_Q19) fill_bgk_sides(kp, k.scalar, s);
+    else if (k.scalar == LBM_SCALAR_Q7) fill_cumulant_sides(kp, s);
 }
 
 cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, float* save,
@@ -553,15 +554,18 @@ cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, flo
     if (k.model == LBM_BGK_SMAG_Q19)
         return launch_bgk_step(kp, k.storage, k.scalar, odd, v, save, trajectory, st);
     if (k.model == LBM_CUMULANT_Q27)
-        return launch_cumulant_step(kp, k.storage, k.scalar, odd, v.f, v.phi, save, st);
+        return launch_cumulant_step(kp, k.storage, k.scalar, odd, v, save, trajectory, st);
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
                          cudaStream_t st) {
     bool ran = false;
-    if (nsteps >= 2 && k.model == LBM_BGK_SMAG_Q19) {
-        const cudaError_t e = launch_bgk_chain(kp, k.storage, k.scalar, odd, nsteps, v, ran, st);
+    if (nsteps >= 2) {
+        const cudaError_t e =
+            k.model == LBM_BGK_SMAG_Q19
+                ? launch_bgk_chain(kp, k.storage, k.scalar, odd, nsteps, v, ran, st)
+                : launch_cumulant_chain(kp, k.storage, k.scalar, odd, nsteps, v, ran, st);
         if (e != cudaSuccess || ran) return e;
     }
     for (int s = 0; s < nsteps; ++s) {

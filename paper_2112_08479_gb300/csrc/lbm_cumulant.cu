@@ -7,8 +7,11 @@
 // collide_cumulant in lbm_cumulant_collide.cuh.
 #include <type_traits>
 
+#include "lbm_chain.cuh"
 #include "lbm_cumulant_collide.cuh"
+#include "lbm_cumulant_lanes.cuh"
 #include "lbm_internal.h"
+#include "lbm_pair.cuh"
 #include "lbm_quad.cuh"
 
 namespace lbmgpu {
@@ -311,6 +314,122 @@ __global__ void __launch_bounds__(128, LBM_CUM_QUAD_MINB)
     even4_body<27, 7, S, Off, CumulantQuadCollide, LBM_CUM_QUAD_NODES>(kp, f, phi);
 }
 
+// FP32 with the D3Q7 scalar: two nodes per thread, x and x + 32
+// (lbm_pair.cuh), one code for both parities, packed arithmetic
+// (lbm_cumulant_lanes.cuh).  428 instructions per node against 621 / 738 of the
+// one-node kernel on even / odd steps; 126 registers without spills, since the
+// inverse stages run in place on the registers of the populations.  One step of
+// 2048x128x256 2.87 -> 2.69 ms (6.8 TB/s, the measured copy rate), 256x32x64 19.8
+// -> 16.6 us.  (The D3Q27 scalar in this form, read twice as in
+// cumulant_fcm_step_body: 13.8 G node updates/s at 1024x64x128 against 14.5, and
+// 11.4 as a chain, whose body of over 24 KB misses the instruction cache; it
+// keeps its one-node kernel.)
+using CumulantTable = PairTable<13, 3, unsigned>;
+
+template <bool EDGE>
+__device__ __forceinline__ void cumulant_pair_step(const KParams& kp, const CumulantTable& tab,
+                                                   float* __restrict__ f, float* __restrict__ phi,
+                                                   bool odd, int x0, int y, int z) {
+    const PairNodes pn = pair_nodes(kp, x0, y, z, odd);
+    const int cls = pair_class(kp, odd, y, z);
+    const size_t fe = (size_t)27 * kp.N, pe = (size_t)7 * kp.N;
+    float2 fv[27], pv[7];
+    pair_gather<13, 0, 27, float, EDGE>(kp, f, pn, tab.f[cls], fv);
+    fv[0] = pair_ld_rest<float, EDGE>(kp, f, fe, pn);
+    pair_gather<3, 0, 7, float, EDGE>(kp, phi, pn, tab.g[cls], pv);
+    pv[0] = pair_ld_rest<float, EDGE>(kp, phi, pe, pn);
+    if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
+        const float s = odd ? 1.0f : -1.0f;   // even steps see the mirrored velocity set
+        collide_cumulant_lanes<Two>(kp, s * kp.gx, s * kp.gy, s * kp.gz, fv, pv);
+    }
+    pair_scatter<3, 0, 7, float, EDGE, false>(kp, phi, pn, tab.g[cls], pv);
+    pair_st_rest<float, EDGE>(kp, phi, pe, pn, pv[0]);
+    pair_scatter<13, 0, 27, float, EDGE, false>(kp, f, pn, tab.f[cls], fv);
+    pair_st_rest<float, EDGE>(kp, f, fe, pn, fv[0]);
+}
+
+__global__ void __launch_bounds__(128, LBM_PAIR_MINB)
+    cumulant_pair_kernel(const __grid_constant__ KParams kp,
+                         const __grid_constant__ CumulantTable tab, float* __restrict__ f,
+                         float* __restrict__ phi, bool odd) {
+    const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (x0 >= kp.nx) return;
+    if (pair_inner(kp, x0))
+        cumulant_pair_step<false>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
+    else
+        cumulant_pair_step<true>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
+}
+
+// Many steps in one launch (lbm_chain.cuh), 14 computing warps of 128 registers.
+// Every segment takes the body that resolves the x ends: a second body for the
+// inner segments costs 116 bytes of spills and instruction cache misses (256x32x64
+// 16.5 us per step against 14.2, 2048x128x256 2.66 ms against 2.48; for the shorter
+// BGK body two are the faster).  Per step, one launch of the former one-node
+// kernel each -> chain: 256x32x64 19.8 -> 14.2 us, 512x64x64 93 -> 61, 1024x64x128
+// 357 -> 269, 2048x128x256 2870 -> 2470 (27.2 G node updates/s).
+constexpr int CUMULANT_CHAIN_WARPS = 14;
+__global__ void __launch_bounds__(32 * (CUMULANT_CHAIN_WARPS + CHAIN_HELPERS), 1)
+    cumulant_chain_kernel(const __grid_constant__ KParams kp, const __grid_constant__ ChainParams cp,
+                          const __grid_constant__ CumulantTable tab, float* __restrict__ f,
+                          float* __restrict__ phi) {
+    chain_run<CUMULANT_CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
+        cumulant_pair_step<true>(kp, tab, f, phi, odd, 64 * seg, y, z);
+    });
+}
+
+cudaError_t launch_cumulant_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
+                                  const Views& v, bool& ran, cudaStream_t st) {
+    ran = false;
+    if (storage != LBM_FP32 || scalar != LBM_SCALAR_Q7 || kp.wide ||
+        (kp.flags & LBM_FLAG_ONE_NODE))
+        return cudaSuccess;
+    ChainPlan pl;
+    cudaError_t e = chain_plan(kp, v, (size_t)kp.nxny * 34 * sizeof(float), 64, CUMULANT_CHAIN_WARPS,
+                               nsteps, odd, pl, ran);
+    if (e != cudaSuccess || !ran) return e;
+    e = cudaMemsetAsync(pl.p.sync, 0, chain_sync_bytes(pl.p), st);
+    if (e != cudaSuccess) return e;
+    cumulant_chain_kernel<<<pl.grid, 32 * (CUMULANT_CHAIN_WARPS + CHAIN_HELPERS), 0, st>>>(
+        kp, pl.p, pair_view<13, 3, unsigned>(*v.sides), (float*)v.f, (float*)v.phi);
+    return cudaGetLastError();
+}
+
+void fill_cumulant_sides(const KParams& kp, Sides& s) {
+    if (!kp.wide) pair_table(kp, 0, pair_view<13, 3, unsigned>(s));   // wide boxes: one node per thread
+}
+
+// One node per thread in the arithmetic of the pairs: LBM_FLAG_ONE_NODE in FP32.
+template <bool ODD>
+__global__ void __launch_bounds__(128) cumulant_node_kernel(KParams kp, float* __restrict__ f,
+                                                            float* __restrict__ phi) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= kp.nx) return;
+    const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
+    float fv[27], pv[7];
+    gather<27, ODD, float>(kp, f, st, fv);
+    gather<7, ODD, float>(kp, phi, st, pv);
+    if (!(kp.flags & LBM_FLAG_NO_COLLIDE))
+        collide_cumulant_lanes<One>(kp, kp.gx, kp.gy, kp.gz, fv, pv);
+    scatter<27, ODD, float>(kp, f, st, fv);
+    scatter<7, ODD, float>(kp, phi, st, pv);
+}
+
+static cudaError_t launch_cumulant_fp32(const KParams& kp, bool odd, const Views& v,
+                                        cudaStream_t st) {
+    float *f = (float*)v.f, *phi = (float*)v.phi;
+    if (kp.flags & LBM_FLAG_ONE_NODE) {
+        dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
+        if (odd) cumulant_node_kernel<true><<<grid, block, 0, st>>>(kp, f, phi);
+        else cumulant_node_kernel<false><<<grid, block, 0, st>>>(kp, f, phi);
+        return cudaGetLastError();
+    }
+    const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
+    dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
+    cumulant_pair_kernel<<<grid, block, 0, st>>>(kp, pair_view<13, 3, unsigned>(*v.sides), f, phi,
+                                                 odd);
+    return cudaGetLastError();
+}
+
 template <typename S, int SL>
 static cudaError_t launch_cumulant_typed(const KParams& kp, bool odd, S* f, S* phi, float* save,
                                         cudaStream_t st) {
@@ -361,10 +480,19 @@ static cudaError_t launch_cumulant_sl(const KParams& kp, int storage, bool odd, 
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd, void* f,
-                                 void* phi, float* save, cudaStream_t st) {
-    if (scalar == LBM_SCALAR_Q7) return launch_cumulant_sl<7>(kp, storage, odd, f, phi, save, st);
-    if (scalar == LBM_SCALAR_Q27) return launch_cumulant_sl<27>(kp, storage, odd, f, phi, save, st);
+// FP32 steps with the D3Q7 scalar take the packed kernels; saved steps and
+// trajectories that the adjoint retraces, boxes with 64-bit offsets, 16-bit
+// storage and the D3Q27 scalar the contracted arithmetic of collide_cumulant
+// (lbm_bgk.cu says why these keep it).
+cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd,
+                                 const Views& v, float* save, bool trajectory, cudaStream_t st) {
+    if (scalar == LBM_SCALAR_Q7) {
+        if (storage == LBM_FP32 && !save && !trajectory && !kp.wide)
+            return launch_cumulant_fp32(kp, odd, v, st);
+        return launch_cumulant_sl<7>(kp, storage, odd, v.f, v.phi, save, st);
+    }
+    if (scalar == LBM_SCALAR_Q27)
+        return launch_cumulant_sl<27>(kp, storage, odd, v.f, v.phi, save, st);
     return cudaErrorInvalidValue;
 }
 

@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 PX, PZ = lbm.LBM_FLAG_PERIODIC_X, lbm.LBM_FLAG_PERIODIC_Z
-KINDS = [(lbm.LBM_BGK_SMAG_Q19, lbm.LBM_SCALAR_Q7), (lbm.LBM_BGK_SMAG_Q19, lbm.LBM_SCALAR_Q6)]
+KINDS = [(lbm.LBM_BGK_SMAG_Q19, lbm.LBM_SCALAR_Q7), (lbm.LBM_BGK_SMAG_Q19, lbm.LBM_SCALAR_Q6),
+         (lbm.LBM_CUMULANT_Q27, lbm.LBM_SCALAR_Q7)]
 W27 = [8 / 27] + [2 / 27] * 6 + [1 / 54] * 12 + [1 / 216] * 8
 WEIGHTS = {19: [1 / 3] + [1 / 18] * 6 + [1 / 36] * 12, 27: W27}
 SCALARS = {7: [1 / 4] + [1 / 8] * 6, 6: [1 / 6] * 6, 27: W27}

@@ -1,4 +1,4 @@
-"""FP32 BGK kernels with two nodes per thread (x and x + 32, packed arithmetic)
+"""FP32 kernels with two nodes per thread (x and x + 32, packed arithmetic)
 against the one-node kernel (LBM_FLAG_ONE_NODE): the collision is written out
 operation by operation and is odd or even under c -> -c, so the states agree
 bit for bit, at segment edges (64 nodes), walls, wraps and extents of one."""
@@ -27,17 +27,19 @@ def _state(p, seed):
     return torch.from_numpy(np.concatenate([f, phi]).astype(np.float32)).cuda()
 
 
-def _params(shape, scalar, flags):
+def _params(shape, kind, flags):
     nx, ny, nz = shape
-    return lbm.Params(nx, ny, nz, scalar=scalar, flags=flags, nu=2e-3, D=3e-3, gprime=1e-4,
+    return lbm.Params(nx, ny, nz, model=kind[0], scalar=kind[1], flags=flags, nu=2e-3, D=3e-3, gprime=1e-4,
                       eg=(0.3, -0.4, -0.866), sc_t=0.7, x0=0, H=nz)
 
 
 @pytest.mark.parametrize("flags", [0, PX, PZ, PX | PZ])
-@pytest.mark.parametrize("scalar", [lbm.LBM_SCALAR_Q7, lbm.LBM_SCALAR_Q6])
+@pytest.mark.parametrize("kind", [(lbm.LBM_BGK_SMAG_Q19, lbm.LBM_SCALAR_Q7),
+                                  (lbm.LBM_BGK_SMAG_Q19, lbm.LBM_SCALAR_Q6),
+                                  (lbm.LBM_CUMULANT_Q27, lbm.LBM_SCALAR_Q7)])
 @pytest.mark.parametrize("shape", SHAPES)
-def test_pair_step_equals_one_node_step(shape, scalar, flags):
-    p = _params(shape, scalar, flags)
+def test_pair_step_equals_one_node_step(shape, kind, flags):
+    p = _params(shape, kind, flags)
     a = lbm.Lattice(p, device="cuda")
     b = lbm.Lattice(dataclasses.replace(p, flags=flags | lbm.LBM_FLAG_ONE_NODE), device="cuda")
     s = _state(p, 11)

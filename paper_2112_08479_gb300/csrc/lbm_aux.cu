@@ -178,7 +178,11 @@ __global__ void set_state_kernel(KParams kp, S* __restrict__ f, S* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// Diagnostics.  One thread per column (x, z), looping over y.
+// Diagnostics.  DIAG_G threads per column (x, z), each summing every DIAG_G-th
+// node along y; their compensated sums are combined in a fixed order.  (One
+// thread per column leaves a small box with one dependent round trip to memory
+// per node of the span and too few warps to hide them: 333x47x59 174 us, DIAGNEW
+// with four; large boxes are bound by reading the state either way.)
 __device__ __forceinline__ unsigned fkey(float v) {
     const unsigned b = __float_as_uint(v);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
@@ -196,21 +200,20 @@ __device__ __forceinline__ void pair_add(float& s, float& c, float t, float d) {
     c = c + d + e;
 }
 
-constexpr int DIAG_BX = 128;
+constexpr int DIAG_BX = 128, DIAG_G = 4;
 
 template <int Q, int SL, bool ODD, typename S>
-__global__ void __launch_bounds__(DIAG_BX) diag_columns_kernel(
+__global__ void __launch_bounds__(DIAG_BX * DIAG_G) diag_columns_kernel(
     KParams kp, const S* __restrict__ f, const S* __restrict__ phi, float* __restrict__ chibar,
     unsigned* __restrict__ colmax, double* __restrict__ part, float* __restrict__ fwpart,
     int* __restrict__ flags) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = threadIdx.x / DIAG_BX, xl = threadIdx.x % DIAG_BX;
+    const int x = blockIdx.x * DIAG_BX + xl;
     const int z = blockIdx.y;
-    double m_rho = 0.0, m_chi = 0.0;
-    float fs = 0.0f, fc = 0.0f;
+    Kahan kc, kr, ku;
     if (x < kp.nx) {
-        Kahan kc, kr, ku;
         int bad = 0;
-        for (int y = 0; y < kp.ny; ++y) {
+        for (int y = g; y < kp.ny; y += DIAG_G) {
             const unsigned n =
                 (unsigned)x + (unsigned)kp.nx * ((unsigned)y + (unsigned)kp.ny * (unsigned)z);
             float d, ux, uy, uz, c;
@@ -223,6 +226,25 @@ __global__ void __launch_bounds__(DIAG_BX) diag_columns_kernel(
                 bad |= LBM_DEVFLAG_NONFINITE;
         }
         if (bad) atomicOr(flags, bad);
+    }
+    __shared__ Kahan part_c[DIAG_G - 1][DIAG_BX], part_r[DIAG_G - 1][DIAG_BX],
+        part_u[DIAG_G - 1][DIAG_BX];
+    if (g > 0) {
+        part_c[g - 1][xl] = kc;
+        part_r[g - 1][xl] = kr;
+        part_u[g - 1][xl] = ku;
+    }
+    __syncthreads();
+    if (g > 0) return;
+#pragma unroll
+    for (int i = 0; i < DIAG_G - 1; ++i) {
+        pair_add(kc.s, kc.c, part_c[i][xl].s, part_c[i][xl].c);
+        pair_add(kr.s, kr.c, part_r[i][xl].s, part_r[i][xl].c);
+        pair_add(ku.s, ku.c, part_u[i][xl].s, part_u[i][xl].c);
+    }
+    double m_rho = 0.0, m_chi = 0.0;
+    float fs = 0.0f, fc = 0.0f;
+    if (x < kp.nx) {
         const float cb = 1.0f + (kc.s + kc.c) / (float)kp.ny;
         chibar[(size_t)z * kp.nx + x] = cb;
         atomicMax(colmax + x, fkey(cb));
@@ -230,11 +252,11 @@ __global__ void __launch_bounds__(DIAG_BX) diag_columns_kernel(
         m_chi = (double)kc.s + (double)kc.c;
         if (kp.nz >= 2 && z < 2) {
             const float a = z == 0 ? 3.0f * kp.nu : -kp.nu * (1.0f / 3.0f);
-            fs = a * ku.s;
-            fc = a * ku.c;
+            scaled_sum(a, ku, fs, fc);
         }
     }
-    // block reductions: budgets in FP64, friction in compensated FP32 pairs
+    // block reductions over the columns (the first DIAG_BX threads): budgets in
+    // FP64, friction in compensated FP32 pairs
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         m_rho += __shfl_down_sync(0xffffffffu, m_rho, o);
@@ -247,7 +269,7 @@ __global__ void __launch_bounds__(DIAG_BX) diag_columns_kernel(
     __shared__ float ss[DIAG_BX / 32], se[DIAG_BX / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) { sr[wid] = m_rho; sc[wid] = m_chi; ss[wid] = fs; se[wid] = fc; }
-    __syncthreads();
+    asm volatile("bar.sync 1, %0;" ::"n"(DIAG_BX) : "memory");
     if (threadIdx.x == 0) {
         double a = 0.0, b = 0.0;
         float s = 0.0f, c = 0.0f;
@@ -622,10 +644,10 @@ cudaError_t launch_diag(const KParams& kp, Kind k, bool odd, const Views& v, dou
     return dispatch(k, [&]<int Q, int SL, typename S>() {
         dim3 grid((kp.nx + DIAG_BX - 1) / DIAG_BX, kp.nz);
         if (odd)
-            diag_columns_kernel<Q, SL, true, S><<<grid, DIAG_BX, 0, st>>>(
+            diag_columns_kernel<Q, SL, true, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
                 kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
         else
-            diag_columns_kernel<Q, SL, false, S><<<grid, DIAG_BX, 0, st>>>(
+            diag_columns_kernel<Q, SL, false, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
                 kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -682,10 +704,10 @@ cudaError_t launch_column_max(const KParams& kp, Kind k, bool odd, const Views& 
     cudaError_t e = dispatch(k, [&]<int Q, int SL, typename S>() {
         dim3 grid((kp.nx + DIAG_BX - 1) / DIAG_BX, kp.nz);
         if (odd)
-            diag_columns_kernel<Q, SL, true, S><<<grid, DIAG_BX, 0, st>>>(
+            diag_columns_kernel<Q, SL, true, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
                 kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
         else
-            diag_columns_kernel<Q, SL, false, S><<<grid, DIAG_BX, 0, st>>>(
+            diag_columns_kernel<Q, SL, false, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
                 kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
         return cudaGetLastError();
     });

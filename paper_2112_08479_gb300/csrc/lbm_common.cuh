@@ -472,4 +472,10 @@ struct Kahan {
     }
 };
 
+// a times the sum, the rounding of the product kept in the low part.
+__device__ __forceinline__ void scaled_sum(float a, const Kahan& k, float& s, float& c) {
+    s = __fmul_rn(a, k.s);
+    c = __fmaf_rn(a, k.c, __fmaf_rn(a, k.s, -s));
+}
+
 }  // namespace lbmgpu

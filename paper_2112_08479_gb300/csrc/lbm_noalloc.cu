@@ -119,8 +119,7 @@ __global__ void __launch_bounds__(NA_BX) na_columns_kernel(KParams kp, const flo
         m_chi = (double)kc.s + (double)kc.c;
         if (kp.nz >= 2 && z < 2) {
             const float a = z == 0 ? 3.0f * kp.nu : -kp.nu * (1.0f / 3.0f);
-            fs = a * ku.s;
-            fc = a * ku.c;
+            scaled_sum(a, ku, fs, fc);
         }
     }
 #pragma unroll

@@ -179,10 +179,14 @@ __global__ void set_state_kernel(KParams kp, S* __restrict__ f, S* __restrict__ 
 
 // ---------------------------------------------------------------------------
 // Diagnostics.  DIAG_G threads per column (x, z), each summing every DIAG_G-th
-// node along y; their compensated sums are combined in a fixed order.  (One
+// node along y; their compensated sums are combined in a fixed order.  One
 // thread per column leaves a small box with one dependent round trip to memory
-// per node of the span and too few warps to hide them: 333x47x59 174 us, DIAGNEW
-// with four; large boxes are bound by reading the state either way.)
+// per node of the span and too few warps to hide them (333x47x59: 118 / 54 us per
+// pass at even / odd parity, 25 / 37 with four; 256x32x64 with the D3Q27 scalar
+// 215 / 84, 27 / 29); a large one is bound by reading the state (2048x128x256
+// FP32 BGK 1109 / 1106 us, 1012 / 1049 with four; FP16 968 / 1015, 741 / 989).
+// The loop over y stays rolled: as the compiler unrolled it, FP16 2048x128x256
+// with four threads took 1683 us at even parity, with two 1894.
 __device__ __forceinline__ unsigned fkey(float v) {
     const unsigned b = __float_as_uint(v);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
@@ -200,10 +204,10 @@ __device__ __forceinline__ void pair_add(float& s, float& c, float t, float d) {
     c = c + d + e;
 }
 
-constexpr int DIAG_BX = 128, DIAG_G = 4;
+constexpr int DIAG_BX = 128;
 
-template <int Q, int SL, bool ODD, typename S>
-__global__ void __launch_bounds__(DIAG_BX * DIAG_G) diag_columns_kernel(
+template <int Q, int SL, bool ODD, typename S, int DIAG_G>
+__global__ void __launch_bounds__(DIAG_BX * DIAG_G, Q == 19 ? 2 : 1) diag_columns_kernel(
     KParams kp, const S* __restrict__ f, const S* __restrict__ phi, float* __restrict__ chibar,
     unsigned* __restrict__ colmax, double* __restrict__ part, float* __restrict__ fwpart,
     int* __restrict__ flags) {
@@ -213,6 +217,7 @@ __global__ void __launch_bounds__(DIAG_BX * DIAG_G) diag_columns_kernel(
     Kahan kc, kr, ku;
     if (x < kp.nx) {
         int bad = 0;
+#pragma unroll 1
         for (int y = g; y < kp.ny; y += DIAG_G) {
             const unsigned n =
                 (unsigned)x + (unsigned)kp.nx * ((unsigned)y + (unsigned)kp.ny * (unsigned)z);
@@ -227,20 +232,22 @@ __global__ void __launch_bounds__(DIAG_BX * DIAG_G) diag_columns_kernel(
         }
         if (bad) atomicOr(flags, bad);
     }
-    __shared__ Kahan part_c[DIAG_G - 1][DIAG_BX], part_r[DIAG_G - 1][DIAG_BX],
-        part_u[DIAG_G - 1][DIAG_BX];
-    if (g > 0) {
-        part_c[g - 1][xl] = kc;
-        part_r[g - 1][xl] = kr;
-        part_u[g - 1][xl] = ku;
-    }
-    __syncthreads();
-    if (g > 0) return;
+    if constexpr (DIAG_G > 1) {
+        __shared__ Kahan part_c[DIAG_G - 1][DIAG_BX], part_r[DIAG_G - 1][DIAG_BX],
+            part_u[DIAG_G - 1][DIAG_BX];
+        if (g > 0) {
+            part_c[g - 1][xl] = kc;
+            part_r[g - 1][xl] = kr;
+            part_u[g - 1][xl] = ku;
+        }
+        __syncthreads();
+        if (g > 0) return;
 #pragma unroll
-    for (int i = 0; i < DIAG_G - 1; ++i) {
-        pair_add(kc.s, kc.c, part_c[i][xl].s, part_c[i][xl].c);
-        pair_add(kr.s, kr.c, part_r[i][xl].s, part_r[i][xl].c);
-        pair_add(ku.s, ku.c, part_u[i][xl].s, part_u[i][xl].c);
+        for (int i = 0; i < DIAG_G - 1; ++i) {
+            pair_add(kc.s, kc.c, part_c[i][xl].s, part_c[i][xl].c);
+            pair_add(kr.s, kr.c, part_r[i][xl].s, part_r[i][xl].c);
+            pair_add(ku.s, ku.c, part_u[i][xl].s, part_u[i][xl].c);
+        }
     }
     double m_rho = 0.0, m_chi = 0.0;
     float fs = 0.0f, fc = 0.0f;
@@ -639,16 +646,26 @@ cudaError_t launch_set_state(const KParams& kp, Kind k, const Views& v, const fl
     });
 }
 
+template <int Q, int SL, typename S>
+static void launch_diag_columns(const KParams& kp, bool odd, const Views& v, cudaStream_t st) {
+    const dim3 grid((kp.nx + DIAG_BX - 1) / DIAG_BX, kp.nz);
+    auto run = [&](auto kernel, int group) {
+        kernel<<<grid, DIAG_BX * group, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, v.chibar,
+                                                 v.colmax, v.part, v.fwpart, v.devflags);
+    };
+    // the odd gather of the 27-velocity fluid prefers fewer rows at a time once the
+    // columns alone fill the chip (2048x128x256 FP32 / FP16: four 1542 / 1418 us, two
+    // 1491 / 1313; 1024x128x128, half of the limit: 402 / 373 and 404 / 363)
+    const bool many = (size_t)kp.nx * kp.nz >= (size_t)1 << 18;
+    if (!odd) run(diag_columns_kernel<Q, SL, false, S, 4>, 4);
+    else if (Q == 27 && many) run(diag_columns_kernel<Q, SL, true, S, Q == 27 ? 2 : 4>, 2);
+    else run(diag_columns_kernel<Q, SL, true, S, 4>, 4);
+}
+
 cudaError_t launch_diag(const KParams& kp, Kind k, bool odd, const Views& v, double threshold,
                         int x0, double H, cudaStream_t st) {
     return dispatch(k, [&]<int Q, int SL, typename S>() {
-        dim3 grid((kp.nx + DIAG_BX - 1) / DIAG_BX, kp.nz);
-        if (odd)
-            diag_columns_kernel<Q, SL, true, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
-                kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
-        else
-            diag_columns_kernel<Q, SL, false, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
-                kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
+        launch_diag_columns<Q, SL, S>(kp, odd, v, st);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         diag_finalize_kernel<<<1, FIN_T, 0, st>>>(kp.nx, (double)kp.N, v.diag_blocks, v.part,
@@ -702,13 +719,7 @@ __global__ void __launch_bounds__(FIN_T) front_of_columns_kernel(const float* __
 cudaError_t launch_column_max(const KParams& kp, Kind k, bool odd, const Views& v, float* m,
                               cudaStream_t st) {
     cudaError_t e = dispatch(k, [&]<int Q, int SL, typename S>() {
-        dim3 grid((kp.nx + DIAG_BX - 1) / DIAG_BX, kp.nz);
-        if (odd)
-            diag_columns_kernel<Q, SL, true, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
-                kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
-        else
-            diag_columns_kernel<Q, SL, false, S><<<grid, DIAG_BX * DIAG_G, 0, st>>>(
-                kp, (const S*)v.f, (const S*)v.phi, v.chibar, v.colmax, v.part, v.fwpart, v.devflags);
+        launch_diag_columns<Q, SL, S>(kp, odd, v, st);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;

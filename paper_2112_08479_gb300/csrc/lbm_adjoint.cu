@@ -18,6 +18,8 @@ namespace lbmgpu {
 __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_push_kernel(KParams kp,
                                                                       const float* __restrict__ src,
                                                                       float* __restrict__ dst) {
+    step_begin();
+    src = ordered(src);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
@@ -67,6 +69,8 @@ __device__ __forceinline__ void bgk_push2_body(const KParams& kp, const float* _
 __global__ void __launch_bounds__(128, LBM_STEP2_MINB) bgk_push2_kernel(KParams kp,
                                                                       const float* __restrict__ src,
                                                                       float* __restrict__ dst) {
+    step_begin();
+    src = ordered(src);
     const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const Stencil2 st = make_stencil2(kp, x, blockIdx.y, blockIdx.z);
     const int z = blockIdx.z;
@@ -80,11 +84,11 @@ __global__ void __launch_bounds__(128, LBM_STEP2_MINB) bgk_push2_kernel(KParams 
 cudaError_t launch_push_step(const KParams& kp, const float* src, float* dst, cudaStream_t st) {
     if (kp.nx % 2 == 0) {
         dim3 block(128), grid((kp.nx / 2 + 127) / 128, kp.ny, kp.nz);
-        bgk_push2_kernel<<<grid, block, 0, st>>>(kp, src, dst);
+        launch_after(bgk_push2_kernel, grid, block, st, kp, src, dst);
         return cudaGetLastError();
     }
     dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-    bgk_push_kernel<<<grid, block, 0, st>>>(kp, src, dst);
+    launch_after(bgk_push_kernel, grid, block, st, kp, src, dst);
     return cudaGetLastError();
 }
 
@@ -109,6 +113,9 @@ __global__ void __launch_bounds__(128, LBM_ADJ_MINB) bgk_adjoint_kernel(KParams 
                                                           float* __restrict__ lam,
                                                           double* __restrict__ dcs, float wfw,
                                                           float dAdCs) {
+    step_begin();
+    st = ordered(st);
+    lamn = ordered(lamn);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     const bool active = x < kp.nx;
@@ -322,7 +329,7 @@ __global__ void __launch_bounds__(128, LBM_ADJ_MINB) bgk_adjoint_kernel(KParams 
 cudaError_t launch_adjoint_step(const KParams& kp, const float* state, const float* lam_next,
                                 float* lam, double* dcs, float wfw, float dAdCs, cudaStream_t st) {
     dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-    bgk_adjoint_kernel<<<grid, block, 0, st>>>(kp, state, lam_next, lam, dcs, wfw, dAdCs);
+    launch_after(bgk_adjoint_kernel, grid, block, st, kp, state, lam_next, lam, dcs, wfw, dAdCs);
     return cudaGetLastError();
 }
 

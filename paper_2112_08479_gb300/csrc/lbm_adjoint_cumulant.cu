@@ -39,6 +39,8 @@ namespace lbmgpu {
 #endif
 __global__ void LBM_CUM_PUSH_BOUNDS cumulant_push_kernel(KParams kp, const float* __restrict__ src,
                                                             float* __restrict__ dst) {
+    step_begin();
+    src = ordered(src);
     using Off = LBM_CUM_PUSH_OFF;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
@@ -55,7 +57,7 @@ __global__ void LBM_CUM_PUSH_BOUNDS cumulant_push_kernel(KParams kp, const float
 cudaError_t launch_cumulant_push_step(const KParams& kp, const float* src, float* dst,
                                       cudaStream_t st) {
     dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-    cumulant_push_kernel<<<grid, block, 0, st>>>(kp, src, dst);
+    launch_after(cumulant_push_kernel, grid, block, st, kp, src, dst);
     return cudaGetLastError();
 }
 
@@ -95,6 +97,9 @@ __device__ __forceinline__ void axis_inverse_vjp(float s, float v, float d0, flo
 __global__ void __launch_bounds__(128, LBM_CUM_ADJ_MINB) cumulant_adjoint_kernel(KParams kp, const float* __restrict__ st,
                                                                const float* __restrict__ lamn,
                                                                float* __restrict__ lam, float wfw) {
+    step_begin();
+    st = ordered(st);
+    lamn = ordered(lamn);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -311,7 +316,7 @@ cudaError_t launch_cumulant_adjoint_step(const KParams& kp, const float* state,
                                          const float* lam_next, float* lam, float wfw,
                                          cudaStream_t st) {
     dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-    cumulant_adjoint_kernel<<<grid, block, 0, st>>>(kp, state, lam_next, lam, wfw);
+    launch_after(cumulant_adjoint_kernel, grid, block, st, kp, state, lam_next, lam, wfw);
     return cudaGetLastError();
 }
 

@@ -118,6 +118,9 @@ template <int Q, int SL, bool ODD, typename S>
 __global__ void macros_kernel(KParams kp, const S* __restrict__ f, const S* __restrict__ phi,
                               float* __restrict__ rho, float* __restrict__ u,
                               float* __restrict__ chi) {
+    step_begin();
+    f = ordered(f);
+    phi = ordered(phi);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -133,6 +136,9 @@ __global__ void macros_kernel(KParams kp, const S* __restrict__ f, const S* __re
 template <int Q, int SL, bool ODD, typename S>
 __global__ void get_state_kernel(KParams kp, const S* __restrict__ f, const S* __restrict__ phi,
                                  float* __restrict__ dst) {
+    step_begin();
+    f = ordered(f);
+    phi = ordered(phi);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -295,6 +301,9 @@ __global__ void __launch_bounds__(FIN_T) diag_finalize_kernel(
     int nx, double nodes, unsigned nblocks, const double* __restrict__ part,
     const float* __restrict__ fwpart, unsigned* __restrict__ colmax, DevDiag* __restrict__ out,
     double thr, int x0, double H, int xlim, int x_off) {
+    step_begin();
+    part = ordered(part);
+    fwpart = ordered(fwpart);
     __shared__ double sa[FIN_T], sb[FIN_T];
     __shared__ float ss[FIN_T], sc[FIN_T];
     __shared__ int sx[FIN_T];
@@ -347,6 +356,9 @@ template <int Q, int SL, bool ODD, typename S>
 __global__ void __launch_bounds__(128) fw_kernel(KParams kp, const S* __restrict__ f,
                                                  const S* __restrict__ phi, double* __restrict__ acc,
                                                  double weight) {
+    step_begin();
+    f = ordered(f);
+    phi = ordered(phi);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y;
     double v = 0.0;
@@ -620,9 +632,9 @@ cudaError_t launch_macros(const KParams& kp, Kind k, bool odd, const Views& v, f
                           float* u, float* chi, cudaStream_t st) {
     return dispatch(k, [&]<int Q, int SL, typename S>() {
         if (odd)
-            macros_kernel<Q, SL, true, S><<<node_grid(kp), 128, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, rho, u, chi);
+            launch_after(macros_kernel<Q, SL, true, S>, node_grid(kp), 128, st, kp, (const S*)v.f, (const S*)v.phi, rho, u, chi);
         else
-            macros_kernel<Q, SL, false, S><<<node_grid(kp), 128, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, rho, u, chi);
+            launch_after(macros_kernel<Q, SL, false, S>, node_grid(kp), 128, st, kp, (const S*)v.f, (const S*)v.phi, rho, u, chi);
         return cudaGetLastError();
     });
 }
@@ -631,9 +643,9 @@ cudaError_t launch_get_state(const KParams& kp, Kind k, bool odd, const Views& v
                              cudaStream_t st) {
     return dispatch(k, [&]<int Q, int SL, typename S>() {
         if (odd)
-            get_state_kernel<Q, SL, true, S><<<node_grid(kp), 128, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, dst);
+            launch_after(get_state_kernel<Q, SL, true, S>, node_grid(kp), 128, st, kp, (const S*)v.f, (const S*)v.phi, dst);
         else
-            get_state_kernel<Q, SL, false, S><<<node_grid(kp), 128, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, dst);
+            launch_after(get_state_kernel<Q, SL, false, S>, node_grid(kp), 128, st, kp, (const S*)v.f, (const S*)v.phi, dst);
         return cudaGetLastError();
     });
 }
@@ -668,7 +680,7 @@ cudaError_t launch_diag(const KParams& kp, Kind k, bool odd, const Views& v, dou
         launch_diag_columns<Q, SL, S>(kp, odd, v, st);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        diag_finalize_kernel<<<1, FIN_T, 0, st>>>(kp.nx, (double)kp.N, v.diag_blocks, v.part,
+        launch_after(diag_finalize_kernel, 1, FIN_T, st, kp.nx, (double)kp.N, v.diag_blocks, v.part,
                                                   v.fwpart, v.colmax, v.ddiag, threshold, x0, H,
                                                   front_xlim(kp.nx, x0, kp.flags), kp.x_off);
         return cudaGetLastError();
@@ -739,9 +751,9 @@ cudaError_t launch_fw_accumulate(const KParams& kp, Kind k, bool odd, const View
     return dispatch(k, [&]<int Q, int SL, typename S>() {
         dim3 grid((kp.nx + 127) / 128, kp.ny);
         if (odd)
-            fw_kernel<Q, SL, true, S><<<grid, 128, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, acc, weight);
+            launch_after(fw_kernel<Q, SL, true, S>, grid, 128, st, kp, (const S*)v.f, (const S*)v.phi, acc, weight);
         else
-            fw_kernel<Q, SL, false, S><<<grid, 128, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, acc, weight);
+            launch_after(fw_kernel<Q, SL, false, S>, grid, 128, st, kp, (const S*)v.f, (const S*)v.phi, acc, weight);
         return cudaGetLastError();
     });
 }

@@ -44,6 +44,7 @@ template <bool ODD, bool SAVE, typename S, int SL, typename Off = unsigned, bool
 __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_step_kernel(KParams kp, S* __restrict__ f,
                                                        S* __restrict__ phi,
                                                        float* __restrict__ save) {
+    step_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
     bgk_pair_kernel(const __grid_constant__ KParams kp,
                     const __grid_constant__ PairTable<9, 3, Off> tab, float* __restrict__ f,
                     float* __restrict__ phi, bool odd) {
+    step_begin();
     const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (x0 >= kp.nx) return;
     if (pair_inner(kp, x0))
@@ -165,6 +167,7 @@ template <bool ODD, bool SAVE, typename S, int SL, typename Off = unsigned>
 __global__ void __launch_bounds__(128, std::is_same<S, float>::value ? LBM_STEP2_MINB : LBM_STEP2_MINB16) bgk_step2_kernel(KParams kp, S* __restrict__ f,
                                                                     S* __restrict__ phi,
                                                                     float* __restrict__ save) {
+    step_begin();
     const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const Stencil2 st = make_stencil2(kp, x, blockIdx.y, blockIdx.z);
     const int z = blockIdx.z;
@@ -201,6 +204,7 @@ struct BgkQuadCollide {
 template <typename S, int SL, typename Off = unsigned>
 __global__ void __launch_bounds__(128, LBM_STEP4_MINB) bgk_even4_kernel(KParams kp, S* __restrict__ f,
                                                                        S* __restrict__ phi) {
+    step_begin();
     even4_body<19, SL, S, Off, BgkQuadCollide>(kp, f, phi);
 }
 
@@ -265,28 +269,28 @@ static cudaError_t launch_bgk_contracted(const KParams& kp, bool odd, S* f, S* p
     if ((kp.flags & LBM_FLAG_ONE_NODE) || kp.nx % 2) {
         dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
         if (save) {
-            if (odd) bgk_step_kernel<true, true, S, SL, unsigned, true><<<grid, block, 0, st>>>(kp, f, phi, save);
-            else bgk_step_kernel<false, true, S, SL, unsigned, true><<<grid, block, 0, st>>>(kp, f, phi, save);
+            if (odd) launch_after(bgk_step_kernel<true, true, S, SL, unsigned, true>, grid, block, st, kp, f, phi, save);
+            else launch_after(bgk_step_kernel<false, true, S, SL, unsigned, true>, grid, block, st, kp, f, phi, save);
         } else {
-            if (odd) bgk_step_kernel<true, false, S, SL, Off, true><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-            else bgk_step_kernel<false, false, S, SL, Off, true><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+            if (odd) launch_after(bgk_step_kernel<true, false, S, SL, Off, true>, grid, block, st, kp, f, phi, nullptr);
+            else launch_after(bgk_step_kernel<false, false, S, SL, Off, true>, grid, block, st, kp, f, phi, nullptr);
         }
         return cudaGetLastError();
     }
     if constexpr (!std::is_same<S, float>::value) {
         if (!odd && !save && kp.nx % 4 == 0) {
             dim3 block(128), grid((kp.nx / 4 + 127) / 128, kp.ny, kp.nz);
-            bgk_even4_kernel<S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi);
+            launch_after(bgk_even4_kernel<S, SL, Off>, grid, block, st, kp, f, phi);
             return cudaGetLastError();
         }
     }
     dim3 block(128), grid((kp.nx / 2 + 127) / 128, kp.ny, kp.nz);
     if (save) {
-        if (odd) bgk_step2_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-        else bgk_step2_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+        if (odd) launch_after(bgk_step2_kernel<true, true, S, SL>, grid, block, st, kp, f, phi, save);
+        else launch_after(bgk_step2_kernel<false, true, S, SL>, grid, block, st, kp, f, phi, save);
     } else {
-        if (odd) bgk_step2_kernel<true, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-        else bgk_step2_kernel<false, false, S, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        if (odd) launch_after(bgk_step2_kernel<true, false, S, SL, Off>, grid, block, st, kp, f, phi, nullptr);
+        else launch_after(bgk_step2_kernel<false, false, S, SL, Off>, grid, block, st, kp, f, phi, nullptr);
     }
     return cudaGetLastError();
 }
@@ -296,13 +300,13 @@ static cudaError_t launch_bgk_fp32(const KParams& kp, const Sides& sides, bool o
                                    float* phi, cudaStream_t st) {
     if (kp.flags & LBM_FLAG_ONE_NODE) {
         dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-        if (odd) bgk_step_kernel<true, false, float, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-        else bgk_step_kernel<false, false, float, SL, Off><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        if (odd) launch_after(bgk_step_kernel<true, false, float, SL, Off>, grid, block, st, kp, f, phi, nullptr);
+        else launch_after(bgk_step_kernel<false, false, float, SL, Off>, grid, block, st, kp, f, phi, nullptr);
         return cudaGetLastError();
     }
     const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
     dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
-    bgk_pair_kernel<SL, Off><<<grid, block, 0, st>>>(kp, pair_view<9, 3, Off>(sides), f, phi, odd);
+    launch_after(bgk_pair_kernel<SL, Off>, grid, block, st, kp, pair_view<9, 3, Off>(sides), f, phi, odd);
     return cudaGetLastError();
 }
 

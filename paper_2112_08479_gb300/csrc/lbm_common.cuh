@@ -455,6 +455,45 @@ __device__ __forceinline__ float csqrt(float x) {
 }
 
 // ---------------------------------------------------------------------------
+// Kernels of consecutive steps overlap their launches (programmatic dependent
+// launch): launched by launch_after, a kernel may become resident while the one
+// before it in the stream drains; step_begin lets its own successor do the same
+// and then waits until the kernel before has completed and its writes are
+// visible.  Every kernel launched so calls step_begin before its first access
+// to global memory.  (Launched in the ordinary way, step_begin does nothing.)
+// What bounds a one-launch step of a small box is the gap between two launches
+// (about 2.3 us of drain and launch, the same at every size): FP16 BGK per step
+// 128x8x16 6.2 -> 4.1 us, 256x32x64 17.5 -> 15.2, 1024x64x128 189.8 -> 187.3,
+// 2048x128x256 1399.7 -> 1397.6; FP16 cumulant 256x32x64 23.4 -> 20.8; one FP32
+// BGK step followed by lbm_macros on 128x8x16 9.2 -> 5.5.
+// A pointer to const that is __restrict__ goes through `ordered` after it: loads
+// through such a pointer may count as invariant and be moved in front of the wait.
+__device__ __forceinline__ void step_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename T>
+__device__ __forceinline__ const T* ordered(const T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st,
+                                A... args) {
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = st;
+    c.attrs = a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Error-free transformation used by the compensated FP32 sums.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = __fadd_rn(a, b);

@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(128, SL == 27 ? (ODD || SAVE ? LBM_Q27_MINB : 
     cumulant_step_kernel(KParams kp, S* __restrict__ f,
                                                             S* __restrict__ phi,
                                                             float* __restrict__ save) {
+    step_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
@@ -311,6 +312,7 @@ struct CumulantQuadCollide {
 template <typename S, typename Off>
 __global__ void __launch_bounds__(128, LBM_CUM_QUAD_MINB)
     cumulant_even4_kernel(KParams kp, S* __restrict__ f, S* __restrict__ phi) {
+    step_begin();
     even4_body<27, 7, S, Off, CumulantQuadCollide, LBM_CUM_QUAD_NODES>(kp, f, phi);
 }
 
@@ -352,6 +354,7 @@ __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
     cumulant_pair_kernel(const __grid_constant__ KParams kp,
                          const __grid_constant__ CumulantTable tab, float* __restrict__ f,
                          float* __restrict__ phi, bool odd) {
+    step_begin();
     const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (x0 >= kp.nx) return;
     if (pair_inner(kp, x0))
@@ -425,7 +428,7 @@ static cudaError_t launch_cumulant_fp32(const KParams& kp, bool odd, const Views
     }
     const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
     dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
-    cumulant_pair_kernel<<<grid, block, 0, st>>>(kp, pair_view<13, 3, unsigned>(*v.sides), f, phi,
+    launch_after(cumulant_pair_kernel, grid, block, st, kp, pair_view<13, 3, unsigned>(*v.sides), f, phi,
                                                  odd);
     return cudaGetLastError();
 }
@@ -438,9 +441,9 @@ static cudaError_t launch_cumulant_typed(const KParams& kp, bool odd, S* f, S* p
         if (!odd && !save && kp.nx % QN == 0 && !(kp.flags & LBM_FLAG_ONE_NODE)) {
             dim3 block(128), grid((kp.nx / QN + 127) / 128, kp.ny, kp.nz);
             if (kp.wide)
-                cumulant_even4_kernel<S, size_t><<<grid, block, 0, st>>>(kp, f, phi);
+                launch_after(cumulant_even4_kernel<S, size_t>, grid, block, st, kp, f, phi);
             else
-                cumulant_even4_kernel<S, LBM_CUM_QUAD_OFF><<<grid, block, 0, st>>>(kp, f, phi);
+                launch_after(cumulant_even4_kernel<S, LBM_CUM_QUAD_OFF>, grid, block, st, kp, f, phi);
             return cudaGetLastError();
         }
     }
@@ -449,19 +452,19 @@ static cudaError_t launch_cumulant_typed(const KParams& kp, bool odd, S* f, S* p
     constexpr bool wide_even = SL == 27 ? LBM_Q27_WIDE_EVEN : LBM_CUM_WIDE_EVEN;
     if (kp.wide) {   // (Q + NS) N >= 2^32: 64-bit element offsets; no saved steps
         if (save) return cudaErrorInvalidValue;
-        if (odd) cumulant_step_kernel<true, false, S, SL, size_t><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
-        else cumulant_step_kernel<false, false, S, SL, size_t><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        if (odd) launch_after(cumulant_step_kernel<true, false, S, SL, size_t>, grid, block, st, kp, f, phi, nullptr);
+        else launch_after(cumulant_step_kernel<false, false, S, SL, size_t>, grid, block, st, kp, f, phi, nullptr);
         return cudaGetLastError();
     }
     if (save) {
-        if (odd) cumulant_step_kernel<true, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
-        else cumulant_step_kernel<false, true, S, SL><<<grid, block, 0, st>>>(kp, f, phi, save);
+        if (odd) launch_after(cumulant_step_kernel<true, true, S, SL>, grid, block, st, kp, f, phi, save);
+        else launch_after(cumulant_step_kernel<false, true, S, SL>, grid, block, st, kp, f, phi, save);
     } else if (odd) {
-        cumulant_step_kernel<true, false, S, SL><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        launch_after(cumulant_step_kernel<true, false, S, SL>, grid, block, st, kp, f, phi, nullptr);
     } else if constexpr (wide_even) {
-        cumulant_step_kernel<false, false, S, SL, size_t><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        launch_after(cumulant_step_kernel<false, false, S, SL, size_t>, grid, block, st, kp, f, phi, nullptr);
     } else {
-        cumulant_step_kernel<false, false, S, SL><<<grid, block, 0, st>>>(kp, f, phi, nullptr);
+        launch_after(cumulant_step_kernel<false, false, S, SL>, grid, block, st, kp, f, phi, nullptr);
     }
     return cudaGetLastError();
 }

@@ -372,10 +372,11 @@ def timed_loop(lat, steps, warmup, torch, inner=INNER, with_diag=True, kernel_ev
     total = t0.elapsed_time(t1) / 1e3
     kern = sum(a.elapsed_time(b) for a, b in evs) / 1e3 / (steps * inner)
     # FP32 steps of one call share a launch (a whole box; slabs step one by one),
-    # except with the D3Q27 scalar
+    # except with the D3Q27 scalar: whole sweeps of three steps on the bench box,
+    # the rest one by one
     chained = (getattr(lat, "peer", None) is None and lat.params.storage == 0
                and lat.params.scalar != 2)
-    launches = steps * ((1 if chained else inner) + (2 if with_diag else 0))
+    launches = steps * ((1 + inner % 3 if chained else inner) + (2 if with_diag else 0))
     return total, kern, launches
 
 

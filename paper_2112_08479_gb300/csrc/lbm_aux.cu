@@ -391,7 +391,7 @@ __global__ void adjoint_chi0_kernel(unsigned N, int Q, const float* __restrict__
 
 // Rules of the chain (lbm_chain.cuh).
 cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, unsigned unit_nodes,
-                       unsigned warps, int nsteps, bool odd, ChainPlan& out, bool& ran) {
+                       unsigned warps, int nsteps, bool odd, ChainPlan& out, int& done) {
     // A box whose state stays in L2 needs no wave: steps in turn, one slot.
     constexpr double RESIDENT = 70e6;
     // Otherwise four slots where the planes between the first and the last one
@@ -407,12 +407,17 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     // (2.5 per computing warp group: published, polled and drawn items): 1.5,
     // 2, 2.5, 3 measured 262, 210, 199, 198 us at 1024x64x128.
     constexpr double SLACK = 2.5;
-    ran = false;
+    done = 0;
     ChainParams& p = out.p;
     const bool resident = plane_bytes * (double)kp.nz <= RESIDENT;
-    // a single step gains nothing, a few steps of a small box not the reset of
-    // the counters (about two launches' worth)
-    if (nsteps < (resident ? 4 : 2)) return cudaSuccess;
+    // Steps that pay for the reset of the counters, the launch and the ramp (14 us on
+    // a box that fits L2), against one overlapped launch per step (launch_after), us
+    // per step: BGK 256x32x64 (55 MB) 16 steps 11.06, 24 10.87, 50 10.54 against
+    // 11.07; cumulant 256x32x64 (71 MB) 16 steps 15.40, 24 14.83 against 14.81;
+    // BGK 333x47x59 (96 MB) 8 steps 26.45, 12 25.14 against 26.00; 512x64x32 (109
+    // MB) 2 steps 31.0 against 31.9; 1024x64x128 2 steps 202 against 253.
+    const double state = plane_bytes * (double)kp.nz;
+    if (nsteps < (state < 80e6 ? 24 : (state < 105e6 ? 12 : 2))) return cudaSuccess;
     if (!resident && (kp.flags & LBM_FLAG_PERIODIC_Z)) return cudaSuccess;   // a wave needs an end
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -420,14 +425,14 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     if (e != cudaSuccess) return e;
     const unsigned nx = (unsigned)kp.nx, ny = (unsigned)kp.ny, nz = (unsigned)kp.nz;
     p.sync = reinterpret_cast<unsigned*>(v.stage);
-    p.nsteps = nsteps;
     p.odd0 = odd ? 1 : 0;
     p.ns = (nx + unit_nodes - 1) / unit_nodes;
-    // units per item: as many as keep the feeding warp ahead of the others, but
-    // no fewer items than there are warps to share them (128x8x16: 3.9 us per
-    // step with 1, 4.4 with 2, 5.1 with 4; 256x32x16: 8.6, 4.8, 5.1)
-    const double units = (double)p.ns * ny * nz;
-    p.U = units < 0.5 * sms * warps ? 1 : (units < 2.0 * sms * warps ? 2 : 4);
+    // units per item: as many as keep the feeding warp ahead of the others (8: no
+    // faster).  A box with fewer than two units per computing warp is done in one
+    // wave of a launch (BGK 256x32x32 8.5 us per step against 6.6, 128x8x16 3.9
+    // against 2.7; past the line 256x32x40 6.8 against 7.9).
+    p.U = 4;
+    if ((double)p.ns * ny * nz < 2.0 * sms * warps) return cudaSuccess;
     int T = resident ? 1 : (nsteps < SLOTS ? nsteps : SLOTS);
     unsigned M, bpt, P, sw, nslab;
     for (;; --T) {
@@ -448,6 +453,11 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     }
     if (T == 1 && !resident) return cudaSuccess;   // too few planes for a wave
     if (CHAIN_COUNTERS + (size_t)P > kp.N) return cudaSuccess;
+    // whole sweeps of T steps; the rest is another call's (a sweep with idle slots
+    // costs a whole one: cumulant 1024x64x128 with three slots, 4 steps 1415 us, 3
+    // steps and one 1166)
+    if (nsteps > T) nsteps -= nsteps % T;
+    p.nsteps = nsteps;
     p.T = T;
     p.groups = (unsigned)((nsteps + T - 1) / T) * nslab;
     const double total = ((double)p.groups * P + (double)(T - 1) * p.lag) * T * bpt;
@@ -461,7 +471,7 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     p.sw.set(sw);
     p.Ud.set(p.U);
     out.grid = (unsigned)sms < p.total ? (unsigned)sms : p.total;
-    ran = true;
+    done = nsteps;
     return cudaSuccess;
 }
 
@@ -601,13 +611,14 @@ cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, flo
 
 cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
                          cudaStream_t st) {
-    bool ran = false;
-    if (nsteps >= 2) {
+    for (int done = 0; nsteps >= 2; nsteps -= done) {
         const cudaError_t e =
             k.model == LBM_BGK_SMAG_Q19
-                ? launch_bgk_chain(kp, k.storage, k.scalar, odd, nsteps, v, ran, st)
-                : launch_cumulant_chain(kp, k.storage, k.scalar, odd, nsteps, v, ran, st);
-        if (e != cudaSuccess || ran) return e;
+                ? launch_bgk_chain(kp, k.storage, k.scalar, odd, nsteps, v, done, st)
+                : launch_cumulant_chain(kp, k.storage, k.scalar, odd, nsteps, v, done, st);
+        if (e != cudaSuccess) return e;
+        if (!done) break;
+        odd ^= (done & 1) != 0;
     }
     for (int s = 0; s < nsteps; ++s) {
         const cudaError_t e = launch_step(kp, k, odd != ((s & 1) != 0), v, nullptr, false, st);

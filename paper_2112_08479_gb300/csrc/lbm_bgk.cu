@@ -232,12 +232,12 @@ __global__ void __launch_bounds__(32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 1)
 }
 
 template <int SL>
-static cudaError_t chain_typed(const KParams& kp, bool odd, int nsteps, const Views& v, bool& ran,
+static cudaError_t chain_typed(const KParams& kp, bool odd, int nsteps, const Views& v, int& done,
                                cudaStream_t st) {
     ChainPlan pl;
     cudaError_t e = chain_plan(kp, v, (size_t)kp.nxny * (19 + ScalarLat<SL>::NS) * sizeof(float), 64,
-                               BGK_CHAIN_WARPS, nsteps, odd, pl, ran);
-    if (e != cudaSuccess || !ran) return e;
+                               BGK_CHAIN_WARPS, nsteps, odd, pl, done);
+    if (e != cudaSuccess || !done) return e;
     e = cudaMemsetAsync(pl.p.sync, 0, chain_sync_bytes(pl.p), st);
     if (e != cudaSuccess) return e;
     bgk_chain_kernel<SL><<<pl.grid, 32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 0, st>>>(
@@ -246,11 +246,11 @@ static cudaError_t chain_typed(const KParams& kp, bool odd, int nsteps, const Vi
 }
 
 cudaError_t launch_bgk_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
-                             const Views& v, bool& ran, cudaStream_t st) {
-    ran = false;
+                             const Views& v, int& done, cudaStream_t st) {
+    done = 0;
     if (storage != LBM_FP32 || kp.wide || (kp.flags & LBM_FLAG_ONE_NODE)) return cudaSuccess;
-    return scalar == LBM_SCALAR_Q7 ? chain_typed<7>(kp, odd, nsteps, v, ran, st)
-                                   : chain_typed<6>(kp, odd, nsteps, v, ran, st);
+    return scalar == LBM_SCALAR_Q7 ? chain_typed<7>(kp, odd, nsteps, v, done, st)
+                                   : chain_typed<6>(kp, odd, nsteps, v, done, st);
 }
 
 // The steps in the contracted arithmetic: every 16-bit step, and in FP32 the

@@ -297,7 +297,7 @@ __device__ __forceinline__ void chain_run(const KParams& kp, const ChainParams& 
 
 // Host side.  Plans a chain of nsteps steps (lbm_aux.cu): plane_bytes of state
 // per plane, units of unit_nodes nodes, `warps` computing warps per block.
-// ran: false when the steps are better launched one by one.  The counters lie
+// done: the steps planned (whole sweeps), 0 when they are better launched one by one.  The counters lie
 // in the staging buffer of lbm_set_scalar (its contents are not kept between
 // calls) and are zeroed on the stream before each launch.
 struct ChainPlan {
@@ -305,7 +305,7 @@ struct ChainPlan {
     unsigned grid;
 };
 cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, unsigned unit_nodes,
-                       unsigned warps, int nsteps, bool odd, ChainPlan& out, bool& ran);
+                       unsigned warps, int nsteps, bool odd, ChainPlan& out, int& done);
 inline size_t chain_sync_bytes(const ChainParams& p) {
     return (CHAIN_COUNTERS + (size_t)p.P.d) * sizeof(unsigned);
 }

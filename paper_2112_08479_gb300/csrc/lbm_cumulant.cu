@@ -381,15 +381,15 @@ __global__ void __launch_bounds__(32 * (CUMULANT_CHAIN_WARPS + CHAIN_HELPERS), 1
 }
 
 cudaError_t launch_cumulant_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
-                                  const Views& v, bool& ran, cudaStream_t st) {
-    ran = false;
+                                  const Views& v, int& done, cudaStream_t st) {
+    done = 0;
     if (storage != LBM_FP32 || scalar != LBM_SCALAR_Q7 || kp.wide ||
         (kp.flags & LBM_FLAG_ONE_NODE))
         return cudaSuccess;
     ChainPlan pl;
     cudaError_t e = chain_plan(kp, v, (size_t)kp.nxny * 34 * sizeof(float), 64, CUMULANT_CHAIN_WARPS,
-                               nsteps, odd, pl, ran);
-    if (e != cudaSuccess || !ran) return e;
+                               nsteps, odd, pl, done);
+    if (e != cudaSuccess || !done) return e;
     e = cudaMemsetAsync(pl.p.sync, 0, chain_sync_bytes(pl.p), st);
     if (e != cudaSuccess) return e;
     cumulant_chain_kernel<<<pl.grid, 32 * (CUMULANT_CHAIN_WARPS + CHAIN_HELPERS), 0, st>>>(

@@ -56,3 +56,18 @@ def test_small_boxes(shape, kind, flags):
 def test_waves_and_slabs(shape, steps, kind):
     _check(shape, kind, 0, steps, steps % 2)
     _check(shape, kind, PX, steps, 0)
+
+
+@pytest.mark.parametrize("flags", [0, PX, PZ])
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("shape", [(3, 66, 66), (65, 33, 70), (129, 41, 37), (256, 32, 48)])
+def test_boxes_in_l2(shape, kind, flags):
+    """Enough rows and steps for one slot, with an odd count from either parity."""
+    _check(shape, kind, flags, 25, 0)
+    _check(shape, kind, flags, 24, 1)
+
+
+@pytest.mark.parametrize("steps", [2, 3, 4, 5, 6, 7, 11])
+@pytest.mark.parametrize("kind", KINDS)
+def test_whole_sweeps_and_the_rest(kind, steps):
+    _check((513, 61, 70), kind, 0, steps, steps % 2)

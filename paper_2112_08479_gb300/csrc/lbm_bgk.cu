@@ -213,9 +213,10 @@ __global__ void __launch_bounds__(128, LBM_STEP4_MINB) bgk_even4_kernel(KParams 
 // against 39 G node updates/s at 2048x128x256).  The body has to be small: with
 // the former step kernels inlined (four bodies of 17 to 20 KB) the mixed
 // parities missed the instruction cache (3.3 of 11.6 cycles per issue) and ran
-// at 26 G.  Per step, one launch each -> chain: 128x8x16 4.4 -> 3.9 us,
-// 256x32x64 12.8 -> 10.1, 333x47x59 28.8 -> 23.3, 1024x64x128 256 -> 183,
-// 2048x128x256 2050 -> 1690 (39.6 G node updates/s, 8.2 TB/s of populations).
+// at 26 G.  Per step, one overlapped launch each -> chain: 256x32x64
+// 11.1 -> 10.5 us, 333x47x59 25.9 -> 23.2, 1024x64x128 252 -> 183, 2048x128x256
+// 2050 -> 1680 (39.9 G node updates/s, 8.3 TB/s of populations); boxes of fewer
+// rows are faster one launch at a time (chain_plan).
 constexpr int BGK_CHAIN_WARPS = 14;
 template <int SL>
 __global__ void __launch_bounds__(32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 1)

@@ -221,6 +221,8 @@ LBM_API lbm_status lbm_set_scalar(lbm_ctx* ctx, const float* chi0);
 /* Advances nsteps >= 0 time steps (Eq. 17), each a fused in-place stream +
  * collide pass (AA pattern: even steps collide in place, odd steps gather from
  * and scatter to the neighbours); the steps of one call may share a launch.
+ * When a launch fails (LBM_ERR_CUDA) the steps launched before it count: the
+ * context's step counter and layout parity are those of the state they leave.
  * Asynchronous. */
 LBM_API lbm_status lbm_step(lbm_ctx* ctx, int32_t nsteps);
 

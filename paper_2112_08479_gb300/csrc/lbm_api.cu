@@ -284,10 +284,13 @@ lbm_status lbm_step(lbm_ctx* c, int32_t nsteps) {
     const Range range("lbm_step");
     if (!c) return arg_fail(nullptr, "ctx is NULL");
     if (nsteps < 0) return arg_fail(c, "nsteps must be >= 0");
-    const cudaError_t e = launch_steps(c->kp, kind(&c->p), c->odd != 0, nsteps, c->v, c->stream);
+    int enqueued = 0;
+    const cudaError_t e =
+        launch_steps(c->kp, kind(&c->p), c->odd != 0, nsteps, c->v, enqueued, c->stream);
+    // the steps that were launched count, also when a later launch failed
+    c->odd ^= enqueued & 1;
+    c->step += enqueued;
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
-    c->odd ^= nsteps & 1;
-    c->step += nsteps;
     return LBM_OK;
 }
 

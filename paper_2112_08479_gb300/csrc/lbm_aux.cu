@@ -16,6 +16,7 @@
 
 #include "lbm_chain.cuh"
 #include "lbm_internal.h"
+#include "lbm_steps.h"
 
 namespace lbmgpu {
 
@@ -610,21 +611,15 @@ cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, flo
 }
 
 cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
-                         cudaStream_t st) {
-    for (int done = 0; nsteps >= 2; nsteps -= done) {
-        const cudaError_t e =
-            k.model == LBM_BGK_SMAG_Q19
-                ? launch_bgk_chain(kp, k.storage, k.scalar, odd, nsteps, v, done, st)
-                : launch_cumulant_chain(kp, k.storage, k.scalar, odd, nsteps, v, done, st);
-        if (e != cudaSuccess) return e;
-        if (!done) break;
-        odd ^= (done & 1) != 0;
-    }
-    for (int s = 0; s < nsteps; ++s) {
-        const cudaError_t e = launch_step(kp, k, odd != ((s & 1) != 0), v, nullptr, false, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+                         int& enqueued, cudaStream_t st) {
+    return enqueue_steps(
+        odd, nsteps, enqueued,
+        [&](bool o, int n, int& done) {
+            return k.model == LBM_BGK_SMAG_Q19
+                       ? launch_bgk_chain(kp, k.storage, k.scalar, o, n, v, done, st)
+                       : launch_cumulant_chain(kp, k.storage, k.scalar, o, n, v, done, st);
+        },
+        [&](bool o) { return launch_step(kp, k, o, v, nullptr, false, st); });
 }
 
 cudaError_t launch_init(const KParams& kp, Kind k, const Views& v, const float* chi0, int x0,

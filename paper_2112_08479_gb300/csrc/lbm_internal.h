@@ -77,9 +77,10 @@ void fill_sides(const KParams& kp, Kind k, Sides& s);
 // (lbm_objective_forward; saved steps always are).
 cudaError_t launch_step(const KParams& kp, Kind k, bool odd, const Views& v, float* save,
                         bool trajectory, cudaStream_t st);
-// nsteps steps, the first of parity `odd`.
+// nsteps steps, the first of parity `odd`; `enqueued` counts those launched, also
+// when a later launch fails (lbm_steps.h).
 cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
-                         cudaStream_t st);
+                         int& enqueued, cudaStream_t st);
 cudaError_t launch_init(const KParams& kp, Kind k, const Views& v, const float* chi0, int x0,
                         double amp, uint64_t seed, cudaStream_t st);
 cudaError_t launch_macros(const KParams& kp, Kind k, bool odd, const Views& v, float* rho,

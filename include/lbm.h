@@ -226,6 +226,19 @@ LBM_API lbm_status lbm_set_scalar(lbm_ctx* ctx, const float* chi0);
  * Asynchronous. */
 LBM_API lbm_status lbm_step(lbm_ctx* ctx, int32_t nsteps);
 
+/* How lbm_step(ctx, nsteps) would begin for a box p on a device of sm_count
+ * multiprocessors: what decides the route, for tests and for reading profiles.
+ * Host only: no device, no context.  out[0] = steps that share the first launch,
+ * 0 when the steps are launched one by one; when not 0, out[1] = step slots (steps
+ * in flight, T), out[2] = slabs along x, out[3] = sweeps through the box, out[4] =
+ * tiles per plane, out[5] = rows per tile, out[6] = items per tile, out[7] = warp
+ * units per item, out[8] = segments of 64 nodes per row, out[9] = segments per row
+ * and slab, out[10] = tiles that a slot runs behind the one before, out[11] =
+ * tickets; else 0.  LBM_ERR_ARG (message in lbm_last_error(NULL)) for an invalid p,
+ * sm_count < 1, nsteps < 0 or a NULL out. */
+LBM_API lbm_status lbm_step_plan(const lbm_params* p, int32_t sm_count, int32_t nsteps,
+                                 int64_t out[12]);
+
 /* One time step that also writes the pre-collision state of the current
  * step, in the canonical layout, to state_out ((Q + NS) * N floats, device).
  * Used to record the forward trajectory for the adjoint: in FP32 it advances

@@ -10,6 +10,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "lbm_chain.cuh"
 #include "lbm_internal.h"
 
 using namespace lbmgpu;
@@ -291,6 +292,23 @@ lbm_status lbm_step(lbm_ctx* c, int32_t nsteps) {
     c->odd ^= enqueued & 1;
     c->step += enqueued;
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+    return LBM_OK;
+}
+
+lbm_status lbm_step_plan(const lbm_params* p, int32_t sm_count, int32_t nsteps, int64_t out[12]) {
+    const char* m = check(p);
+    if (!m && sm_count < 1) m = "sm_count must be >= 1";
+    if (!m && nsteps < 0) m = "nsteps must be >= 0";
+    if (!m && !out) m = "out is NULL";
+    if (m) return arg_fail(nullptr, m);
+    ChainPlan pl = {};
+    const ChainParams& c = pl.p;
+    const int done = chain_plan(kparams(p), kind(p), (unsigned)sm_count, nsteps, false, pl);
+    memset(out, 0, 12 * sizeof out[0]);
+    if (!done) return LBM_OK;
+    const int64_t v[12] = {done, c.T, c.nslab.d, c.groups / c.nslab.d, c.M.d, c.R, c.bpt.d,
+                           c.U, c.ns, c.sw.d, c.lag, c.total};
+    memcpy(out, v, sizeof v);
     return LBM_OK;
 }
 

@@ -391,8 +391,13 @@ __global__ void adjoint_chi0_kernel(unsigned N, int Q, const float* __restrict__
 }
 
 // Rules of the chain (lbm_chain.cuh).
-cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, unsigned unit_nodes,
-                       unsigned warps, int nsteps, bool odd, ChainPlan& out, int& done) {
+int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, ChainPlan& out) {
+    if (k.storage != LBM_FP32 || k.scalar == LBM_SCALAR_Q27 || kp.wide ||
+        (kp.flags & LBM_FLAG_ONE_NODE))
+        return 0;
+    const int rows = (k.model == LBM_CUMULANT_Q27 ? 27 : 19) + (k.scalar == LBM_SCALAR_Q6 ? 6 : 7);
+    const size_t plane_bytes = (size_t)kp.nxny * rows * sizeof(float);
+    constexpr unsigned warps = CHAIN_WARPS;
     // A box whose state stays in L2 needs no wave: steps in turn, one slot.
     constexpr double RESIDENT = 70e6;
     // Otherwise four slots where the planes between the first and the last one
@@ -408,7 +413,6 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     // (2.5 per computing warp group: published, polled and drawn items): 1.5,
     // 2, 2.5, 3 measured 262, 210, 199, 198 us at 1024x64x128.
     constexpr double SLACK = 2.5;
-    done = 0;
     ChainParams& p = out.p;
     const bool resident = plane_bytes * (double)kp.nz <= RESIDENT;
     // Steps that pay for the reset of the counters, the launch and the ramp (14 us on
@@ -418,22 +422,18 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     // BGK 333x47x59 (96 MB) 8 steps 26.45, 12 25.14 against 26.00; 512x64x32 (109
     // MB) 2 steps 31.0 against 31.9; 1024x64x128 2 steps 202 against 253.
     const double state = plane_bytes * (double)kp.nz;
-    if (nsteps < (state < 80e6 ? 24 : (state < 105e6 ? 12 : 2))) return cudaSuccess;
-    if (!resident && (kp.flags & LBM_FLAG_PERIODIC_Z)) return cudaSuccess;   // a wave needs an end
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
+    if (nsteps < (state < 80e6 ? 24 : (state < 105e6 ? 12 : 2))) return 0;
+    if (!resident && (kp.flags & LBM_FLAG_PERIODIC_Z)) return 0;   // a wave needs an end
     const unsigned nx = (unsigned)kp.nx, ny = (unsigned)kp.ny, nz = (unsigned)kp.nz;
-    p.sync = reinterpret_cast<unsigned*>(v.stage);
+    p.sync = nullptr;
     p.odd0 = odd ? 1 : 0;
-    p.ns = (nx + unit_nodes - 1) / unit_nodes;
+    p.ns = (nx + CHAIN_UNIT - 1) / CHAIN_UNIT;
     // units per item: as many as keep the feeding warp ahead of the others (8: no
     // faster).  A box with fewer than two units per computing warp is done in one
     // wave of a launch (BGK 256x32x32 8.5 us per step against 6.6, 128x8x16 3.9
     // against 2.7; past the line 256x32x40 6.8 against 7.9).
     p.U = 4;
-    if ((double)p.ns * ny * nz < 2.0 * sms * warps) return cudaSuccess;
+    if ((double)p.ns * ny * nz < 2.0 * sms * warps) return 0;
     int T = resident ? 1 : (nsteps < SLOTS ? nsteps : SLOTS);
     unsigned M, bpt, P, sw, nslab;
     for (;; --T) {
@@ -452,8 +452,8 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
         if (T > SLOTS_SLABS && live > LIVE) continue;
         if (T == 1 || (double)(T - 1) * p.lag + 2.0 * M <= P) break;
     }
-    if (T == 1 && !resident) return cudaSuccess;   // too few planes for a wave
-    if (CHAIN_COUNTERS + (size_t)P > kp.N) return cudaSuccess;
+    if (T == 1 && !resident) return 0;   // too few planes for a wave
+    if (CHAIN_COUNTERS + (size_t)P > kp.N) return 0;
     // whole sweeps of T steps; the rest is another call's (a sweep with idle slots
     // costs a whole one: cumulant 1024x64x128 with three slots, 4 steps 1415 us, 3
     // steps and one 1166)
@@ -462,7 +462,7 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     p.T = T;
     p.groups = (unsigned)((nsteps + T - 1) / T) * nslab;
     const double total = ((double)p.groups * P + (double)(T - 1) * p.lag) * T * bpt;
-    if (total >= 2147000000.0) return cudaSuccess;   // 31-bit tickets
+    if (total >= 2147000000.0) return 0;   // 31-bit tickets
     p.total = (unsigned)total;
     p.M.set(M);
     p.bpt.set(bpt);
@@ -471,9 +471,21 @@ cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, un
     p.nslab.set(nslab);
     p.sw.set(sw);
     p.Ud.set(p.U);
-    out.grid = (unsigned)sms < p.total ? (unsigned)sms : p.total;
-    done = nsteps;
-    return cudaSuccess;
+    out.grid = sms < p.total ? sms : p.total;
+    return nsteps;
+}
+
+cudaError_t chain_prepare(const KParams& kp, Kind k, const Views& v, int nsteps, bool odd,
+                          ChainPlan& out, int& done, cudaStream_t st) {
+    done = 0;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    done = chain_plan(kp, k, (unsigned)sms, nsteps, odd, out);
+    if (!done) return cudaSuccess;
+    out.p.sync = reinterpret_cast<unsigned*>(v.stage);
+    return cudaMemsetAsync(out.p.sync, 0, (CHAIN_COUNTERS + (size_t)out.p.P.d) * sizeof(unsigned), st);
 }
 
 // ---------------------------------------------------------------------------
@@ -616,8 +628,8 @@ cudaError_t launch_steps(const KParams& kp, Kind k, bool odd, int nsteps, const 
         odd, nsteps, enqueued,
         [&](bool o, int n, int& done) {
             return k.model == LBM_BGK_SMAG_Q19
-                       ? launch_bgk_chain(kp, k.storage, k.scalar, o, n, v, done, st)
-                       : launch_cumulant_chain(kp, k.storage, k.scalar, o, n, v, done, st);
+                       ? launch_bgk_chain(kp, k, o, n, v, done, st)
+                       : launch_cumulant_chain(kp, k, o, n, v, done, st);
         },
         [&](bool o) { return launch_step(kp, k, o, v, nullptr, false, st); });
 }

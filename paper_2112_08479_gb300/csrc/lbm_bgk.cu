@@ -217,13 +217,12 @@ __global__ void __launch_bounds__(128, LBM_STEP4_MINB) bgk_even4_kernel(KParams 
 // 11.1 -> 10.5 us, 333x47x59 25.9 -> 23.2, 1024x64x128 252 -> 183, 2048x128x256
 // 2050 -> 1680 (39.9 G node updates/s, 8.3 TB/s of populations); boxes of fewer
 // rows are faster one launch at a time (chain_plan).
-constexpr int BGK_CHAIN_WARPS = 14;
 template <int SL>
-__global__ void __launch_bounds__(32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 1)
+__global__ void __launch_bounds__(CHAIN_THREADS, 1)
     bgk_chain_kernel(const __grid_constant__ KParams kp, const __grid_constant__ ChainParams cp,
                      const __grid_constant__ PairTable<9, 3, unsigned> tab, float* __restrict__ f,
                      float* __restrict__ phi) {
-    chain_run<BGK_CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
+    chain_run<CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
         const int x0 = 64 * seg;
         if (pair_inner(kp, x0))
             bgk_pair_step<SL, false, unsigned>(kp, tab, f, phi, odd, x0, y, z);
@@ -233,25 +232,19 @@ __global__ void __launch_bounds__(32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 1)
 }
 
 template <int SL>
-static cudaError_t chain_typed(const KParams& kp, bool odd, int nsteps, const Views& v, int& done,
-                               cudaStream_t st) {
-    ChainPlan pl;
-    cudaError_t e = chain_plan(kp, v, (size_t)kp.nxny * (19 + ScalarLat<SL>::NS) * sizeof(float), 64,
-                               BGK_CHAIN_WARPS, nsteps, odd, pl, done);
-    if (e != cudaSuccess || !done) return e;
-    e = cudaMemsetAsync(pl.p.sync, 0, chain_sync_bytes(pl.p), st);
-    if (e != cudaSuccess) return e;
-    bgk_chain_kernel<SL><<<pl.grid, 32 * (BGK_CHAIN_WARPS + CHAIN_HELPERS), 0, st>>>(
+static cudaError_t launch_chain(const KParams& kp, const ChainPlan& pl, const Views& v,
+                                cudaStream_t st) {
+    bgk_chain_kernel<SL><<<pl.grid, CHAIN_THREADS, 0, st>>>(
         kp, pl.p, pair_view<9, 3, unsigned>(*v.sides), (float*)v.f, (float*)v.phi);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bgk_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
-                             const Views& v, int& done, cudaStream_t st) {
-    done = 0;
-    if (storage != LBM_FP32 || kp.wide || (kp.flags & LBM_FLAG_ONE_NODE)) return cudaSuccess;
-    return scalar == LBM_SCALAR_Q7 ? chain_typed<7>(kp, odd, nsteps, v, done, st)
-                                   : chain_typed<6>(kp, odd, nsteps, v, done, st);
+cudaError_t launch_bgk_chain(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
+                             int& done, cudaStream_t st) {
+    ChainPlan pl;
+    const cudaError_t e = chain_prepare(kp, k, v, nsteps, odd, pl, done, st);
+    if (e != cudaSuccess || !done) return e;
+    return k.scalar == LBM_SCALAR_Q7 ? launch_chain<7>(kp, pl, v, st) : launch_chain<6>(kp, pl, v, st);
 }
 
 // The steps in the contracted arithmetic: every 16-bit step, and in FP32 the

@@ -295,19 +295,24 @@ __device__ __forceinline__ void chain_run(const KParams& kp, const ChainParams& 
     }
 }
 
-// Host side.  Plans a chain of nsteps steps (lbm_aux.cu): plane_bytes of state
-// per plane, units of unit_nodes nodes, `warps` computing warps per block.
-// done: the steps planned (whole sweeps), 0 when they are better launched one by one.  The counters lie
-// in the staging buffer of lbm_set_scalar (its contents are not kept between
-// calls) and are zeroed on the stream before each launch.
+// Host side.  Warp units are segments of 64 nodes; 14 computing warps per block
+// at 128 registers (lbm_bgk.cu).
+constexpr int CHAIN_WARPS = 14;
+constexpr int CHAIN_UNIT = 64;
+constexpr int CHAIN_THREADS = 32 * (CHAIN_WARPS + CHAIN_HELPERS);
+
+// Plans a chain of up to nsteps steps on a device of `sms` SMs (lbm_aux.cu); also
+// read by lbm_step_plan.  Returns the steps planned (whole sweeps), 0 when they are
+// better launched one by one or no chain kernel serves the kind of box.
 struct ChainPlan {
-    ChainParams p;
+    ChainParams p;      // p.sync is the launcher's to set
     unsigned grid;
 };
-cudaError_t chain_plan(const KParams& kp, const Views& v, size_t plane_bytes, unsigned unit_nodes,
-                       unsigned warps, int nsteps, bool odd, ChainPlan& out, int& done);
-inline size_t chain_sync_bytes(const ChainParams& p) {
-    return (CHAIN_COUNTERS + (size_t)p.P.d) * sizeof(unsigned);
-}
+int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, ChainPlan& out);
+
+// The plan on the current device, with its counters in the staging buffer of
+// lbm_set_scalar (whose contents are not kept between calls), zeroed on the stream.
+cudaError_t chain_prepare(const KParams& kp, Kind k, const Views& v, int nsteps, bool odd,
+                          ChainPlan& out, int& done, cudaStream_t st);
 
 }  // namespace lbmgpu

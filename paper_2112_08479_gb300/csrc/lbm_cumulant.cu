@@ -370,29 +370,21 @@ __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
 // BGK body two are the faster).  Per step, one launch of the former one-node
 // kernel each -> chain: 256x32x64 19.8 -> 14.2 us, 512x64x64 93 -> 61, 1024x64x128
 // 357 -> 269, 2048x128x256 2870 -> 2470 (27.2 G node updates/s).
-constexpr int CUMULANT_CHAIN_WARPS = 14;
-__global__ void __launch_bounds__(32 * (CUMULANT_CHAIN_WARPS + CHAIN_HELPERS), 1)
+__global__ void __launch_bounds__(CHAIN_THREADS, 1)
     cumulant_chain_kernel(const __grid_constant__ KParams kp, const __grid_constant__ ChainParams cp,
                           const __grid_constant__ CumulantTable tab, float* __restrict__ f,
                           float* __restrict__ phi) {
-    chain_run<CUMULANT_CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
+    chain_run<CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
         cumulant_pair_step<true>(kp, tab, f, phi, odd, 64 * seg, y, z);
     });
 }
 
-cudaError_t launch_cumulant_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
-                                  const Views& v, int& done, cudaStream_t st) {
-    done = 0;
-    if (storage != LBM_FP32 || scalar != LBM_SCALAR_Q7 || kp.wide ||
-        (kp.flags & LBM_FLAG_ONE_NODE))
-        return cudaSuccess;
+cudaError_t launch_cumulant_chain(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
+                                  int& done, cudaStream_t st) {
     ChainPlan pl;
-    cudaError_t e = chain_plan(kp, v, (size_t)kp.nxny * 34 * sizeof(float), 64, CUMULANT_CHAIN_WARPS,
-                               nsteps, odd, pl, done);
+    const cudaError_t e = chain_prepare(kp, k, v, nsteps, odd, pl, done, st);
     if (e != cudaSuccess || !done) return e;
-    e = cudaMemsetAsync(pl.p.sync, 0, chain_sync_bytes(pl.p), st);
-    if (e != cudaSuccess) return e;
-    cumulant_chain_kernel<<<pl.grid, 32 * (CUMULANT_CHAIN_WARPS + CHAIN_HELPERS), 0, st>>>(
+    cumulant_chain_kernel<<<pl.grid, CHAIN_THREADS, 0, st>>>(
         kp, pl.p, pair_view<13, 3, unsigned>(*v.sides), (float*)v.f, (float*)v.phi);
     return cudaGetLastError();
 }

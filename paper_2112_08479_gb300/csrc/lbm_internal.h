@@ -46,23 +46,23 @@ struct Views {
     const Sides* sides;   // host memory of the context
 };
 
-// Per-model step launchers (lbm_bgk.cu, lbm_cumulant.cu).
-void fill_bgk_sides(const KParams& kp, int scalar, Sides& s);
-cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, const Views& v,
-                            float* save, bool trajectory, cudaStream_t st);
-cudaError_t launch_bgk_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
-                             const Views& v, int& done, cudaStream_t st);
-void fill_cumulant_sides(const KParams& kp, Sides& s);
-cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd,
-                                 const Views& v, float* save, bool trajectory, cudaStream_t st);
-cudaError_t launch_cumulant_chain(const KParams& kp, int storage, int scalar, bool odd, int nsteps,
-                                  const Views& v, int& done, cudaStream_t st);
-
 // Model, scalar lattice and storage select the kernel (the pairs the ABI
 // accepts: BGK with D3Q7 or D3Q6, cumulant with D3Q7 or D3Q27).
 struct Kind {
     int model, scalar, storage;
 };
+
+// Per-model step launchers (lbm_bgk.cu, lbm_cumulant.cu).
+void fill_bgk_sides(const KParams& kp, int scalar, Sides& s);
+cudaError_t launch_bgk_step(const KParams& kp, int storage, int scalar, bool odd, const Views& v,
+                            float* save, bool trajectory, cudaStream_t st);
+cudaError_t launch_bgk_chain(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
+                             int& done, cudaStream_t st);
+void fill_cumulant_sides(const KParams& kp, Sides& s);
+cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd,
+                                 const Views& v, float* save, bool trajectory, cudaStream_t st);
+cudaError_t launch_cumulant_chain(const KParams& kp, Kind k, bool odd, int nsteps, const Views& v,
+                                  int& done, cudaStream_t st);
 
 // The TMA-staged step kernels (lbm_staged.cu): whether they serve this box
 // and kind, and their launcher.

@@ -76,6 +76,7 @@ SIGNATURES = [
     ("lbm_init", C.c_int, [_P, C.c_void_p, C.c_size_t, C.c_void_p, C.POINTER(C.c_void_p)]),
     ("lbm_set_scalar", C.c_int, [_CTX, C.c_void_p]),
     ("lbm_step", C.c_int, [_CTX, C.c_int32]),
+    ("lbm_step_plan", C.c_int, [_P, C.c_int32, C.c_int32, C.POINTER(C.c_int64)]),
     ("lbm_step_save", C.c_int, [_CTX, C.c_void_p]),
     ("lbm_macros", C.c_int, [_CTX, C.c_void_p, C.c_void_p, C.c_void_p]),
     ("lbm_diag", C.c_int, [_CTX, C.POINTER(lbm_diagnostics)]),
@@ -168,6 +169,18 @@ def lbm_set_scalar(ctx, chi0_ptr: int):
 
 def lbm_step(ctx, n: int):
     _check(load().lbm_step(ctx, n), ctx)
+
+
+# out[i] of lbm_step_plan
+STEP_PLAN = ("steps", "slots", "slabs", "sweeps", "tiles", "rows", "items", "units", "segments",
+             "slab_segments", "lag", "tickets")
+
+
+def lbm_step_plan(p: lbm_params, sm_count: int, n: int) -> dict:
+    """How lbm_step would begin n steps of the box p on sm_count SMs."""
+    out = (C.c_int64 * 12)()
+    _check(load().lbm_step_plan(C.byref(p), sm_count, n, out))
+    return dict(zip(STEP_PLAN, out))
 
 
 def lbm_step_save(ctx, state_ptr: int):

@@ -12,6 +12,8 @@
 // Column sums run in FP32 with Kahan compensation, block and grid sums of the
 // budgets in FP64, the friction in compensated FP32 pairs; every reduction
 // has a fixed order, so results are bitwise reproducible.
+#include <math.h>
+
 #include <type_traits>
 
 #include "lbm_chain.cuh"
@@ -457,12 +459,18 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
     // whole sweeps of T steps; the rest is another call's (a sweep with idle slots
     // costs a whole one: cumulant 1024x64x128 with three slots, 4 steps 1415 us, 3
     // steps and one 1166)
+    // ... and no more than keep every unit of the launch below 2^31, the range of Div
+    // and of a block's unit counter should one block take all of them: 1,820 steps of
+    // 2048x128x256.  The rest is the next launch's.
+    const double tickets = 2147483648.0 / p.U - 1.0;
+    const double sweeps = floor((tickets / ((double)T * bpt) - (double)(T - 1) * p.lag) / P / nslab);
+    if (sweeps < 1.0) return 0;
     if (nsteps > T) nsteps -= nsteps % T;
+    if (nsteps > sweeps * T) nsteps = (int)(sweeps * T);
     p.nsteps = nsteps;
     p.T = T;
     p.groups = (unsigned)((nsteps + T - 1) / T) * nslab;
     const double total = ((double)p.groups * P + (double)(T - 1) * p.lag) * T * bpt;
-    if (total >= 2147000000.0) return 0;   // 31-bit tickets
     p.total = (unsigned)total;
     p.M.set(M);
     p.bpt.set(bpt);

@@ -140,6 +140,29 @@ def test_bench_box():
     assert (pl["steps"], pl["slots"], pl["slabs"], pl["sweeps"]) == (99, 3, 3, 33)
 
 
+@pytest.mark.parametrize("shape,flags,model", [
+    ((2048, 128, 256), 0, BGK), ((2500, 150, 100), PX, BGK), ((1024, 64, 128), 0, CUM),
+    ((256, 32, 64), PZ, BGK), ((65535, 2, 300), 0, CUM)])
+@pytest.mark.parametrize("steps", [8000, 1000003, 2**31 - 1])
+def test_long_calls_share_launches(shape, flags, model, steps):
+    """A call of any length goes by launches of whole sweeps whose units stay
+    below 2^31; only the steps short of a sweep are left."""
+    short = _plan(shape, 100, flags, model)
+    pl = _plan(shape, steps, flags, model)
+    assert pl["tickets"] * pl["units"] < 2**31 and pl["steps"] <= steps
+    for k in ("slots", "slabs", "tiles", "rows", "items", "lag"):
+        assert pl[k] == short[k]
+    assert pl["steps"] == pl["sweeps"] * pl["slots"]
+    per_sweep = pl["slabs"] * pl["tiles"] * shape[2] * pl["slots"] * pl["items"]
+    if pl["steps"] < steps - steps % pl["slots"]:      # cut: one sweep more does not fit
+        assert (pl["tickets"] + per_sweep) * pl["units"] >= 2**31
+    left, launches = steps, 0
+    while (n := _plan(shape, left, flags, model)["steps"]):
+        k = max(1, left // n - 1)                       # launches of this size in a row
+        left, launches = left - k * n, launches + k
+    assert left < 24 and launches <= steps / 1000 + 8
+
+
 def test_arguments():
     import ctypes as C
     p, out = lbm.Params(64, 4, 8, H=8).c(), (C.c_int64 * 12)()

@@ -479,6 +479,8 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
     p.nslab.set(nslab);
     p.sw.set(sw);
     p.Ud.set(p.U);
+    p.stall = (kp.flags & LBM_FLAG_TEST_STALL) != 0;
+    p.limit_ns = p.stall ? CHAIN_STALL_NS : CHAIN_LIMIT_NS;
     out.grid = sms < p.total ? sms : p.total;
     return nsteps;
 }

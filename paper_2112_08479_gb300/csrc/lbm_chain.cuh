@@ -28,7 +28,10 @@
 // group nu the 3 x 3 tiles around must count nu bpt.  All these have smaller
 // tickets (lag >= M + 3; nz M >= (T - 1) lag + 2 M), and every ticket drawn is
 // held by a running block, so the wait always ends, whatever else runs on the
-// GPU; it is bounded all the same (CHAIN_LIMIT_NS, LBM_DEVFLAG_TIMEOUT).
+// GPU; it is bounded all the same (ChainParams::limit_ns, LBM_DEVFLAG_TIMEOUT): a
+// feeding warp that gives up sets the abort word, which the waits of the other
+// blocks see, and `stop`, after which the computing warps finish what is published
+// and the announcing warp ends with the last of it.
 //
 // Roles.  In each block NW warps compute; a feeding warp draws tickets, waits
 // for their counters (acquire) and publishes ready items in a ring in shared
@@ -74,9 +77,12 @@ struct ChainParams {
     Div nslab;          // x slabs
     Div sw;             // warp segments per row and slab
     Div Ud;             // U
+    unsigned long long limit_ns;   // longest wait for a counter
+    int stall;          // LBM_FLAG_TEST_STALL: the first item of the first tile is not counted
 };
 
 constexpr unsigned long long CHAIN_LIMIT_NS = 10000000000ull;   // only a defect waits that long
+constexpr unsigned long long CHAIN_STALL_NS = 100000000ull;     // the limit under the test hook
 constexpr unsigned CHAIN_COUNTERS = 32;   // first counter in ChainParams::sync (a line of its own)
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
@@ -193,7 +199,7 @@ __device__ __forceinline__ void chain_run(const KParams& kp, const ChainParams& 
         // feeding warp: tickets, dependencies, publication
         const unsigned grp = lane / 9u, k = lane - grp * 9u;   // item of the group, neighbour
         const int dz = (int)(k / 3u) - 1, dy = (int)(k % 3u) - 1;
-        const unsigned long long limit = CHAIN_LIMIT_NS;
+        const unsigned long long limit = cp.limit_ns;
         ChainItem im, nx;
         const unsigned *dep, *ndep;
         // the item of this lane's group in tickets t ..., and the counter of its
@@ -281,7 +287,8 @@ __device__ __forceinline__ void chain_run(const KParams& kp, const ChainParams& 
                 const ChainItem im = sh.item[lane];
                 fence_gpu();
                 if (full) {
-                    red_add(done + ((unsigned)im.z * cp.M.d + (unsigned)im.tile), 1u);
+                    const bool held = cp.stall && (im.nu | im.z | im.tile | im.b) == 0;
+                    if (!held) red_add(done + ((unsigned)im.z * cp.M.d + (unsigned)im.tile), 1u);
                     sh.finished[lane] = 0;
                     ++seen;
                     sts_release(&sh.freed[lane], seen);

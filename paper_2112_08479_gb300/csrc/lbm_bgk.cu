@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(128, LBM_STEP_MINB) bgk_step_kernel(KParams kp
 
 // FP32: two nodes per thread, x and x + 32 (lbm_pair.cuh), one code for both
 // parities, packed arithmetic.
-template <int SL, bool EDGE, typename Off>
-__device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable<9, 3, Off>& tab,
+template <int SL, bool EDGE, bool WIDE>
+__device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable<9, 3>& tab,
                                               float* __restrict__ f, float* __restrict__ phi,
                                               bool odd, int x0, int y, int z) {
     constexpr int NS = ScalarLat<SL>::NS, D0 = ScalarLat<SL>::D0;
@@ -85,32 +85,32 @@ __device__ __forceinline__ void bgk_pair_step(const KParams& kp, const PairTable
     const int cls = pair_class(kp, odd, y, z);
     const size_t fe = (size_t)19 * kp.N, pe = (size_t)NS * kp.N;
     float2 fv[19], pv[NS];
-    pair_gather<9, 0, 19, float, EDGE>(kp, f, pn, tab.f[cls], fv);
-    pair_gather<3, D0, NS, float, EDGE>(kp, phi, pn, tab.g[cls], pv);
+    pair_gather<9, 0, 19, float, EDGE, WIDE>(kp, f, pn, tab.f[cls], fv);
+    pair_gather<3, D0, NS, float, EDGE, WIDE>(kp, phi, pn, tab.g[cls], pv);
     fv[0] = pair_ld_rest<float, EDGE>(kp, f, fe, pn);
     if constexpr (SL == 7) pv[0] = pair_ld_rest<float, EDGE>(kp, phi, pe, pn);
     if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
         const float s = odd ? 1.0f : -1.0f;   // even steps see the mirrored velocity set
         collide_bgk_lanes<Two, SL>(kp, s * kp.gx, s * kp.gy, s * kp.gz, fv, pv);
     }
-    pair_scatter<9, 0, 19, float, EDGE, false>(kp, f, pn, tab.f[cls], fv);
-    pair_scatter<3, D0, NS, float, EDGE, false>(kp, phi, pn, tab.g[cls], pv);
+    pair_scatter<9, 0, 19, float, EDGE, WIDE>(kp, f, pn, tab.f[cls], fv);
+    pair_scatter<3, D0, NS, float, EDGE, WIDE>(kp, phi, pn, tab.g[cls], pv);
     pair_st_rest<float, EDGE>(kp, f, fe, pn, fv[0]);
     if constexpr (SL == 7) pair_st_rest<float, EDGE>(kp, phi, pe, pn, pv[0]);
 }
 
-template <int SL, typename Off>
+template <int SL, bool WIDE>
 __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
     bgk_pair_kernel(const __grid_constant__ KParams kp,
-                    const __grid_constant__ PairTable<9, 3, Off> tab, float* __restrict__ f,
+                    const __grid_constant__ PairTable<9, 3> tab, float* __restrict__ f,
                     float* __restrict__ phi, bool odd) {
     step_begin();
     const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (x0 >= kp.nx) return;
     if (pair_inner(kp, x0))
-        bgk_pair_step<SL, false, Off>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
+        bgk_pair_step<SL, false, WIDE>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
     else
-        bgk_pair_step<SL, true, Off>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
+        bgk_pair_step<SL, true, WIDE>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
 }
 
 #ifndef LBM_BGK_ZSPLIT
@@ -220,14 +220,14 @@ __global__ void __launch_bounds__(128, LBM_STEP4_MINB) bgk_even4_kernel(KParams 
 template <int SL>
 __global__ void __launch_bounds__(CHAIN_THREADS, 1)
     bgk_chain_kernel(const __grid_constant__ KParams kp, const __grid_constant__ ChainParams cp,
-                     const __grid_constant__ PairTable<9, 3, unsigned> tab, float* __restrict__ f,
+                     const __grid_constant__ PairTable<9, 3> tab, float* __restrict__ f,
                      float* __restrict__ phi) {
     chain_run<CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
         const int x0 = 64 * seg;
         if (pair_inner(kp, x0))
-            bgk_pair_step<SL, false, unsigned>(kp, tab, f, phi, odd, x0, y, z);
+            bgk_pair_step<SL, false, false>(kp, tab, f, phi, odd, x0, y, z);
         else
-            bgk_pair_step<SL, true, unsigned>(kp, tab, f, phi, odd, x0, y, z);
+            bgk_pair_step<SL, true, false>(kp, tab, f, phi, odd, x0, y, z);
     });
 }
 
@@ -235,7 +235,7 @@ template <int SL>
 static cudaError_t launch_chain(const KParams& kp, const ChainPlan& pl, const Views& v,
                                 cudaStream_t st) {
     bgk_chain_kernel<SL><<<pl.grid, CHAIN_THREADS, 0, st>>>(
-        kp, pl.p, pair_view<9, 3, unsigned>(*v.sides), (float*)v.f, (float*)v.phi);
+        kp, pl.p, pair_view<9, 3>(*v.sides), (float*)v.f, (float*)v.phi);
     return cudaGetLastError();
 }
 
@@ -289,10 +289,11 @@ static cudaError_t launch_bgk_contracted(const KParams& kp, bool odd, S* f, S* p
     return cudaGetLastError();
 }
 
-template <int SL, typename Off>
+template <int SL, bool WIDE>
 static cudaError_t launch_bgk_fp32(const KParams& kp, const Sides& sides, bool odd, float* f,
                                    float* phi, cudaStream_t st) {
     if (kp.flags & LBM_FLAG_ONE_NODE) {
+        using Off = std::conditional_t<WIDE, size_t, unsigned>;
         dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
         if (odd) launch_after(bgk_step_kernel<true, false, float, SL, Off>, grid, block, st, kp, f, phi, nullptr);
         else launch_after(bgk_step_kernel<false, false, float, SL, Off>, grid, block, st, kp, f, phi, nullptr);
@@ -300,15 +301,12 @@ static cudaError_t launch_bgk_fp32(const KParams& kp, const Sides& sides, bool o
     }
     const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
     dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
-    launch_after(bgk_pair_kernel<SL, Off>, grid, block, st, kp, pair_view<9, 3, Off>(sides), f, phi, odd);
+    launch_after(bgk_pair_kernel<SL, WIDE>, grid, block, st, kp, pair_view<9, 3>(sides), f, phi, odd);
     return cudaGetLastError();
 }
 
 void fill_bgk_sides(const KParams& kp, int scalar, Sides& s) {
-    const int d0 = scalar == LBM_SCALAR_Q6 ? 1 : 0;
-    // 32-bit element offsets unless (Q + NS) N >= 2^32 (KParams::wide)
-    if (kp.wide) pair_table(kp, d0, pair_view<9, 3, size_t>(s));
-    else pair_table(kp, d0, pair_view<9, 3, unsigned>(s));
+    pair_table(kp, scalar == LBM_SCALAR_Q6 ? 1 : 0, pair_view<9, 3>(s));
 }
 
 template <typename S, int SL>
@@ -317,8 +315,8 @@ static cudaError_t launch_bgk_typed(const KParams& kp, bool odd, const Views& v,
     S *f = (S*)v.f, *phi = (S*)v.phi;
     if constexpr (std::is_same<S, float>::value) {
         if (!save && !trajectory)
-            return kp.wide ? launch_bgk_fp32<SL, size_t>(kp, *v.sides, odd, f, phi, st)
-                           : launch_bgk_fp32<SL, unsigned>(kp, *v.sides, odd, f, phi, st);
+            return kp.wide ? launch_bgk_fp32<SL, true>(kp, *v.sides, odd, f, phi, st)
+                           : launch_bgk_fp32<SL, false>(kp, *v.sides, odd, f, phi, st);
     }
     return kp.wide ? launch_bgk_contracted<S, SL, size_t>(kp, odd, f, phi, save, st)
                    : launch_bgk_contracted<S, SL, unsigned>(kp, odd, f, phi, save, st);

@@ -326,9 +326,13 @@ __global__ void __launch_bounds__(128, LBM_CUM_QUAD_MINB)
 // cumulant_fcm_step_body: 13.8 G node updates/s at 1024x64x128 against 14.5, and
 // 11.4 as a chain, whose body of over 24 KB misses the instruction cache; it
 // keeps its one-node kernel.)
-using CumulantTable = PairTable<13, 3, unsigned>;
+// WIDE (64-bit offsets): 72 bytes of spills; the former one-node kernel -> pairs, one
+// step of 2048x256x256 5.76 -> 5.53 ms, 1025x400x330 6.13 -> 6.07, 300x700x650 6.48
+// -> 6.32, 130x1100x1000 7.67 -> 7.71.  (With a 64-bit offset per side and thread: 384
+// bytes, 5.83 ms.)
+using CumulantTable = PairTable<13, 3>;
 
-template <bool EDGE>
+template <bool EDGE, bool WIDE>
 __device__ __forceinline__ void cumulant_pair_step(const KParams& kp, const CumulantTable& tab,
                                                    float* __restrict__ f, float* __restrict__ phi,
                                                    bool odd, int x0, int y, int z) {
@@ -336,20 +340,21 @@ __device__ __forceinline__ void cumulant_pair_step(const KParams& kp, const Cumu
     const int cls = pair_class(kp, odd, y, z);
     const size_t fe = (size_t)27 * kp.N, pe = (size_t)7 * kp.N;
     float2 fv[27], pv[7];
-    pair_gather<13, 0, 27, float, EDGE>(kp, f, pn, tab.f[cls], fv);
+    pair_gather<13, 0, 27, float, EDGE, WIDE>(kp, f, pn, tab.f[cls], fv);
     fv[0] = pair_ld_rest<float, EDGE>(kp, f, fe, pn);
-    pair_gather<3, 0, 7, float, EDGE>(kp, phi, pn, tab.g[cls], pv);
+    pair_gather<3, 0, 7, float, EDGE, WIDE>(kp, phi, pn, tab.g[cls], pv);
     pv[0] = pair_ld_rest<float, EDGE>(kp, phi, pe, pn);
     if (!(kp.flags & LBM_FLAG_NO_COLLIDE)) {
         const float s = odd ? 1.0f : -1.0f;   // even steps see the mirrored velocity set
         collide_cumulant_lanes<Two>(kp, s * kp.gx, s * kp.gy, s * kp.gz, fv, pv);
     }
-    pair_scatter<3, 0, 7, float, EDGE, false>(kp, phi, pn, tab.g[cls], pv);
+    pair_scatter<3, 0, 7, float, EDGE, WIDE>(kp, phi, pn, tab.g[cls], pv);
     pair_st_rest<float, EDGE>(kp, phi, pe, pn, pv[0]);
-    pair_scatter<13, 0, 27, float, EDGE, false>(kp, f, pn, tab.f[cls], fv);
+    pair_scatter<13, 0, 27, float, EDGE, WIDE>(kp, f, pn, tab.f[cls], fv);
     pair_st_rest<float, EDGE>(kp, f, fe, pn, fv[0]);
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
     cumulant_pair_kernel(const __grid_constant__ KParams kp,
                          const __grid_constant__ CumulantTable tab, float* __restrict__ f,
@@ -358,9 +363,9 @@ __global__ void __launch_bounds__(128, LBM_PAIR_MINB)
     const int x0 = 64 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (x0 >= kp.nx) return;
     if (pair_inner(kp, x0))
-        cumulant_pair_step<false>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
+        cumulant_pair_step<false, WIDE>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
     else
-        cumulant_pair_step<true>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
+        cumulant_pair_step<true, WIDE>(kp, tab, f, phi, odd, x0, blockIdx.y, blockIdx.z);
 }
 
 // Many steps in one launch (lbm_chain.cuh), 14 computing warps of 128 registers.
@@ -375,7 +380,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS, 1)
                           const __grid_constant__ CumulantTable tab, float* __restrict__ f,
                           float* __restrict__ phi) {
     chain_run<CHAIN_WARPS>(kp, cp, [&](bool odd, int seg, int y, int z) {
-        cumulant_pair_step<true>(kp, tab, f, phi, odd, 64 * seg, y, z);
+        cumulant_pair_step<true, false>(kp, tab, f, phi, odd, 64 * seg, y, z);
     });
 }
 
@@ -385,43 +390,43 @@ cudaError_t launch_cumulant_chain(const KParams& kp, Kind k, bool odd, int nstep
     const cudaError_t e = chain_prepare(kp, k, v, nsteps, odd, pl, done, st);
     if (e != cudaSuccess || !done) return e;
     cumulant_chain_kernel<<<pl.grid, CHAIN_THREADS, 0, st>>>(
-        kp, pl.p, pair_view<13, 3, unsigned>(*v.sides), (float*)v.f, (float*)v.phi);
+        kp, pl.p, pair_view<13, 3>(*v.sides), (float*)v.f, (float*)v.phi);
     return cudaGetLastError();
 }
 
-void fill_cumulant_sides(const KParams& kp, Sides& s) {
-    if (!kp.wide) pair_table(kp, 0, pair_view<13, 3, unsigned>(s));   // wide boxes: one node per thread
-}
+void fill_cumulant_sides(const KParams& kp, Sides& s) { pair_table(kp, 0, pair_view<13, 3>(s)); }
 
 // One node per thread in the arithmetic of the pairs: LBM_FLAG_ONE_NODE in FP32.
-template <bool ODD>
+template <bool ODD, typename Off>
 __global__ void __launch_bounds__(128) cumulant_node_kernel(KParams kp, float* __restrict__ f,
                                                             float* __restrict__ phi) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
     float fv[27], pv[7];
-    gather<27, ODD, float>(kp, f, st, fv);
-    gather<7, ODD, float>(kp, phi, st, pv);
+    gather<27, ODD, float, 0, false, true, Off>(kp, f, st, fv);
+    gather<7, ODD, float, 0, false, true, Off>(kp, phi, st, pv);
     if (!(kp.flags & LBM_FLAG_NO_COLLIDE))
         collide_cumulant_lanes<One>(kp, kp.gx, kp.gy, kp.gz, fv, pv);
-    scatter<27, ODD, float>(kp, f, st, fv);
-    scatter<7, ODD, float>(kp, phi, st, pv);
+    scatter<27, ODD, float, 0, false, true, Off>(kp, f, st, fv);
+    scatter<7, ODD, float, 0, false, true, Off>(kp, phi, st, pv);
 }
 
+template <bool WIDE>
 static cudaError_t launch_cumulant_fp32(const KParams& kp, bool odd, const Views& v,
                                         cudaStream_t st) {
     float *f = (float*)v.f, *phi = (float*)v.phi;
     if (kp.flags & LBM_FLAG_ONE_NODE) {
+        using Off = std::conditional_t<WIDE, size_t, unsigned>;
         dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-        if (odd) cumulant_node_kernel<true><<<grid, block, 0, st>>>(kp, f, phi);
-        else cumulant_node_kernel<false><<<grid, block, 0, st>>>(kp, f, phi);
+        if (odd) cumulant_node_kernel<true, Off><<<grid, block, 0, st>>>(kp, f, phi);
+        else cumulant_node_kernel<false, Off><<<grid, block, 0, st>>>(kp, f, phi);
         return cudaGetLastError();
     }
     const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
     dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
-    launch_after(cumulant_pair_kernel, grid, block, st, kp, pair_view<13, 3, unsigned>(*v.sides), f, phi,
-                                                 odd);
+    launch_after(cumulant_pair_kernel<WIDE>, grid, block, st, kp, pair_view<13, 3>(*v.sides), f, phi,
+                 odd);
     return cudaGetLastError();
 }
 
@@ -475,15 +480,16 @@ static cudaError_t launch_cumulant_sl(const KParams& kp, int storage, bool odd, 
     return cudaErrorInvalidValue;
 }
 
-// FP32 steps with the D3Q7 scalar take the packed kernels; saved steps and
-// trajectories that the adjoint retraces, boxes with 64-bit offsets, 16-bit
-// storage and the D3Q27 scalar the contracted arithmetic of collide_cumulant
-// (lbm_bgk.cu says why these keep it).
+// FP32 steps with the D3Q7 scalar take the packed kernels (a box with 64-bit offsets
+// too: its x-slabs may have 32-bit ones and have to give the same bits); saved steps
+// and trajectories that the adjoint retraces, 16-bit storage and the D3Q27 scalar
+// the contracted arithmetic of collide_cumulant (lbm_bgk.cu says why these keep it).
 cudaError_t launch_cumulant_step(const KParams& kp, int storage, int scalar, bool odd,
                                  const Views& v, float* save, bool trajectory, cudaStream_t st) {
     if (scalar == LBM_SCALAR_Q7) {
-        if (storage == LBM_FP32 && !save && !trajectory && !kp.wide)
-            return launch_cumulant_fp32(kp, odd, v, st);
+        if (storage == LBM_FP32 && !save && !trajectory)
+            return kp.wide ? launch_cumulant_fp32<true>(kp, odd, v, st)
+                           : launch_cumulant_fp32<false>(kp, odd, v, st);
         return launch_cumulant_sl<7>(kp, storage, odd, v.f, v.phi, save, st);
     }
     if (scalar == LBM_SCALAR_Q27)

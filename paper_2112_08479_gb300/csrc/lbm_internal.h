@@ -27,7 +27,7 @@ struct FrontGrad {
 // a node (lbm_pair.cuh), filled once per context: a host-side buffer that the
 // launchers pass to the kernels by value.
 struct Sides {
-    alignas(16) unsigned char bytes[3264];
+    alignas(16) unsigned char bytes[2176];
 };
 
 // Workspace views handed to the launchers.

@@ -34,11 +34,14 @@ constexpr int PAIR_CLASSES = 17;   // the even step; odd: 1 + 4 (z position) + (
 
 // Element offsets from the node to the sides of the fluid (F opposite pairs)
 // and of the scalar (G opposite pairs): [2 m] is side P of pair m, [2 m + 1]
-// side M; formed modulo 2^32 (or 2^64).
-template <int F, int G, typename Off>
+// side M; formed modulo 2^32.  Arrays of 2^32 elements or more (WIDE,
+// KParams::wide) hold them relative to the first of the pair's two rows, whose
+// 64-bit base is the same for every thread: node and offset then make less than
+// 2 N < 2^32.
+template <int F, int G>
 struct PairTable {
-    Off f[PAIR_CLASSES][2 * F];
-    Off g[PAIR_CLASSES][2 * G];
+    unsigned f[PAIR_CLASSES][2 * F];
+    unsigned g[PAIR_CLASSES][2 * G];
 };
 
 // Position of a coordinate: 0 inside, 1 first, 2 last, 3 both (extent 1).
@@ -48,18 +51,18 @@ __host__ __device__ constexpr int pair_pos(int c, int n) {
 
 // Fills the sides of M opposite pairs of directions 1, 2, ... whose rows are
 // direction - d0.
-template <int M, typename Off>
-inline void pair_sides(const KParams& kp, int d0, Off (&o)[PAIR_CLASSES][2 * M]) {
+template <int M>
+inline void pair_sides(const KParams& kp, int d0, unsigned (&o)[PAIR_CLASSES][2 * M]) {
     const long long N = kp.N;
     const bool pz = (kp.flags & LBM_FLAG_PERIODIC_Z) != 0;
     for (int cls = 0; cls < PAIR_CLASSES; ++cls) {
         const int yp = cls ? (cls - 1) % 4 : 0, zp = cls ? (cls - 1) / 4 : 0;
         for (int m = 0; m < M; ++m) {
-            const int i = 2 * m + 1;
+            const int i = 2 * m + 1, row = kp.wide ? 0 : i - d0;   // of direction i
             for (int side = 0; side < 2; ++side) {
                 const int s = side == 0 ? 1 : -1;   // P: n + c_i, M: n - c_i
-                const long long own = (long long)((side == 0 ? i : i + 1) - d0) * N;
-                const long long other = (long long)((side == 0 ? i + 1 : i) - d0) * N;
+                const long long own = (row + (side == 0 ? 0 : 1)) * N;
+                const long long other = (row + (side == 0 ? 1 : 0)) * N;
                 long long v = own;
                 if (cls) {
                     const int cx = s * cx27(i), cy = s * cy27(i), cz = s * cz27(i);
@@ -73,27 +76,27 @@ inline void pair_sides(const KParams& kp, int d0, Off (&o)[PAIR_CLASSES][2 * M])
                         v += (long long)(cz + (zlo ? kp.nz : (zhi ? -kp.nz : 0))) * kp.nxny;
                     }
                 }
-                o[cls][2 * m + side] = (Off)v;
+                o[cls][2 * m + side] = (unsigned)v;
             }
         }
     }
 }
 
-template <int F, int G, typename Off>
-inline void pair_table(const KParams& kp, int d0, PairTable<F, G, Off>& t) {
-    pair_sides<F, Off>(kp, 0, t.f);
-    pair_sides<G, Off>(kp, d0, t.g);
+template <int F, int G>
+inline void pair_table(const KParams& kp, int d0, PairTable<F, G>& t) {
+    pair_sides<F>(kp, 0, t.f);
+    pair_sides<G>(kp, d0, t.g);
 }
 
 // The context's copy (Sides), as the type it was filled with.
-template <int F, int G, typename Off>
-inline PairTable<F, G, Off>& pair_view(Sides& s) {
-    static_assert(sizeof(PairTable<F, G, Off>) <= sizeof s.bytes);
-    return *reinterpret_cast<PairTable<F, G, Off>*>(s.bytes);
+template <int F, int G>
+inline PairTable<F, G>& pair_view(Sides& s) {
+    static_assert(sizeof(PairTable<F, G>) <= sizeof s.bytes);
+    return *reinterpret_cast<PairTable<F, G>*>(s.bytes);
 }
-template <int F, int G, typename Off>
-inline const PairTable<F, G, Off>& pair_view(const Sides& s) {
-    return pair_view<F, G, Off>(const_cast<Sides&>(s));
+template <int F, int G>
+inline const PairTable<F, G>& pair_view(const Sides& s) {
+    return pair_view<F, G>(const_cast<Sides&>(s));
 }
 
 // Warps of a block along x (of ns 64-node segments per row): as many, up to
@@ -146,82 +149,91 @@ __device__ __forceinline__ bool pair_inner(const KParams& kp, int x0) {
 // opposite direction (row `other`) at a wall (as the table has it already
 // where the side meets a z wall), the wrapped column with periodic ends.
 // dx, dz: the side's displacement.
-template <typename Off>
-__host__ __device__ __forceinline__ Off pair_edge(const KParams& kp, const PairNodes& pn, int x,
-                                                  Off off, int other, int dx, int dz) {
+__host__ __device__ __forceinline__ unsigned pair_edge(const KParams& kp, const PairNodes& pn,
+                                                       int x, unsigned off, unsigned other, int dx,
+                                                       int dz) {
     // (selects, no branches: the loads that follow must not wait for each other)
     const bool turned = (dz < 0 && (pn.zwall & 1)) || (dz > 0 && (pn.zwall & 2));
-    const Off alt = (kp.flags & LBM_FLAG_PERIODIC_X) ? off - (Off)(long long)(dx * kp.nx)
-                                                     : (Off)other * kp.N;
+    const unsigned alt = (kp.flags & LBM_FLAG_PERIODIC_X) ? off - (unsigned)(dx * kp.nx)
+                                                          : other * kp.N;
     const bool out = dx < 0 ? x == 0 : (dx > 0 ? x == kp.nx - 1 : false);
     return out && pn.odd && !turned ? alt : off;
 }
 
-// Loads the two nodes' elements of a side.
-template <typename S, bool EDGE, typename Off>
+// The array from which the offsets of the pair with direction i in row `row`
+// count: the array itself, or that row (WIDE).
+template <bool WIDE, typename S>
+__device__ __forceinline__ S* pair_base(const KParams& kp, S* a, int row) {
+    return WIDE ? a + (size_t)row * kp.N : a;
+}
+
+// Loads the two nodes' elements of a side, at offsets from `base` (in array a).
+template <typename S, bool EDGE>
 __device__ __forceinline__ float2 pair_ld(const KParams& kp, const S* __restrict__ a, size_t extent,
-                                          const PairNodes& pn, Off off, int other, int dx, int dz) {
+                                          const S* base, const PairNodes& pn, unsigned off,
+                                          int other, int dx, int dz) {
     float2 v = make_float2(0.0f, 0.0f);
     if constexpr (!EDGE) {
-        const Off e = (Off)pn.n + off;
-        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, a + e, 1, extent)) v.x = Store<S>::ld(a + e);
-        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, a + e + 32, 1, extent)) v.y = Store<S>::ld(a + e + 32);
+        const unsigned e = pn.n + off;
+        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, base + e, 1, extent)) v.x = Store<S>::ld(base + e);
+        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, base + e + 32, 1, extent)) v.y = Store<S>::ld(base + e + 32);
     } else {
         // lanes beyond the row read what the last node reads, and drop it: the
         // loads stay unconditional, so none waits for the one before
-        const Off e0 = (Off)pn.clamped(kp, 0) + pair_edge(kp, pn, min(pn.x, kp.nx - 1), off, other, dx, dz);
-        const Off e1 = (Off)pn.clamped(kp, 32) + pair_edge(kp, pn, min(pn.x + 32, kp.nx - 1), off, other, dx, dz);
-        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, a + e0, 1, extent)) v.x = Store<S>::ld(a + e0);
-        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, a + e1, 1, extent)) v.y = Store<S>::ld(a + e1);
+        const unsigned e0 = pn.clamped(kp, 0) + pair_edge(kp, pn, min(pn.x, kp.nx - 1), off, other, dx, dz);
+        const unsigned e1 = pn.clamped(kp, 32) + pair_edge(kp, pn, min(pn.x + 32, kp.nx - 1), off, other, dx, dz);
+        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, base + e0, 1, extent)) v.x = Store<S>::ld(base + e0);
+        if (LBM_IN(kp, LBM_SITE_PAIR_LOAD, a, base + e1, 1, extent)) v.y = Store<S>::ld(base + e1);
     }
     return v;
 }
 
-template <typename S, bool EDGE, typename Off>
-__device__ __forceinline__ void pair_st(const KParams& kp, S* __restrict__ a, size_t extent,
-                                        const PairNodes& pn, Off off, int other, int dx, int dz,
-                                        float2 v) {
+template <typename S, bool EDGE>
+__device__ __forceinline__ void pair_st(const KParams& kp, S* __restrict__ a, size_t extent, S* base,
+                                        const PairNodes& pn, unsigned off, int other, int dx,
+                                        int dz, float2 v) {
     if constexpr (!EDGE) {
-        const Off e = (Off)pn.n + off;
-        if (LBM_IN(kp, LBM_SITE_PAIR_STORE, a, a + e, 1, extent)) Store<S>::st(a + e, v.x);
-        if (LBM_IN(kp, LBM_SITE_PAIR_STORE, a, a + e + 32, 1, extent)) Store<S>::st(a + e + 32, v.y);
+        const unsigned e = pn.n + off;
+        if (LBM_IN(kp, LBM_SITE_PAIR_STORE, a, base + e, 1, extent)) Store<S>::st(base + e, v.x);
+        if (LBM_IN(kp, LBM_SITE_PAIR_STORE, a, base + e + 32, 1, extent)) Store<S>::st(base + e + 32, v.y);
     } else {
-        const Off e0 = (Off)pn.n + pair_edge(kp, pn, pn.x, off, other, dx, dz);
-        const Off e1 = (Off)(pn.n + 32) + pair_edge(kp, pn, pn.x + 32, off, other, dx, dz);
-        if (pn.x < kp.nx && LBM_IN(kp, LBM_SITE_PAIR_STORE, a, a + e0, 1, extent))
-            Store<S>::st(a + e0, v.x);
-        if (pn.x + 32 < kp.nx && LBM_IN(kp, LBM_SITE_PAIR_STORE, a, a + e1, 1, extent))
-            Store<S>::st(a + e1, v.y);
+        const unsigned e0 = pn.n + pair_edge(kp, pn, pn.x, off, other, dx, dz);
+        const unsigned e1 = pn.n + 32 + pair_edge(kp, pn, pn.x + 32, off, other, dx, dz);
+        if (pn.x < kp.nx && LBM_IN(kp, LBM_SITE_PAIR_STORE, a, base + e0, 1, extent))
+            Store<S>::st(base + e0, v.x);
+        if (pn.x + 32 < kp.nx && LBM_IN(kp, LBM_SITE_PAIR_STORE, a, base + e1, 1, extent))
+            Store<S>::st(base + e1, v.y);
     }
 }
 
 // Gather of M opposite pairs (rows direction - D0 of an array of ROWS rows):
 // f_i from side M, f_(i+1) from side P; the rest population is the caller's.
-template <int M, int D0, int ROWS, typename S, bool EDGE, typename Off>
+template <int M, int D0, int ROWS, typename S, bool EDGE, bool WIDE>
 __device__ __forceinline__ void pair_gather(const KParams& kp, const S* __restrict__ a,
-                                            const PairNodes& pn, const Off* off,
+                                            const PairNodes& pn, const unsigned* off,
                                             float2 (&v)[ROWS]) {
     const size_t ext = (size_t)ROWS * kp.N;
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-        const int i = 2 * m + 1, cx = cx27(i), cz = cz27(i);
-        v[i - D0] = pair_ld<S, EDGE>(kp, a, ext, pn, off[2 * m + 1], i - D0, -cx, -cz);
-        v[i + 1 - D0] = pair_ld<S, EDGE>(kp, a, ext, pn, off[2 * m], i + 1 - D0, cx, cz);
+        const int i = 2 * m + 1, cx = cx27(i), cz = cz27(i), row = WIDE ? 0 : i - D0;
+        const S* b = pair_base<WIDE>(kp, a, i - D0);
+        v[i - D0] = pair_ld<S, EDGE>(kp, a, ext, b, pn, off[2 * m + 1], row, -cx, -cz);
+        v[i + 1 - D0] = pair_ld<S, EDGE>(kp, a, ext, b, pn, off[2 * m], row + 1, cx, cz);
     }
 }
 
-// Scatter of the post-collision populations: f*_i to side P, f*_(i+1) to side
-// M (SWAP: the other way round, for values named by the mirrored set).
-template <int M, int D0, int ROWS, typename S, bool EDGE, bool SWAP, typename Off>
+// Scatter of the post-collision populations: f*_i to side P, f*_(i+1) to side M.
+template <int M, int D0, int ROWS, typename S, bool EDGE, bool WIDE>
 __device__ __forceinline__ void pair_scatter(const KParams& kp, S* __restrict__ a,
-                                             const PairNodes& pn, const Off* off,
+                                             const PairNodes& pn, const unsigned* off,
                                              const float2 (&v)[ROWS]) {
     const size_t ext = (size_t)ROWS * kp.N;
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-        const int i = 2 * m + 1, cx = cx27(i), cz = cz27(i);
-        pair_st<S, EDGE>(kp, a, ext, pn, off[2 * m], i + 1 - D0, cx, cz, v[(SWAP ? i + 1 : i) - D0]);
-        pair_st<S, EDGE>(kp, a, ext, pn, off[2 * m + 1], i - D0, -cx, -cz, v[(SWAP ? i : i + 1) - D0]);
+        const int i = 2 * m + 1, cx = cx27(i), cz = cz27(i), row = WIDE ? 0 : i - D0;
+        S* b = pair_base<WIDE>(kp, a, i - D0);
+        pair_st<S, EDGE>(kp, a, ext, b, pn, off[2 * m], row + 1, cx, cz, v[i - D0]);
+        pair_st<S, EDGE>(kp, a, ext, b, pn, off[2 * m + 1], row, -cx, -cz, v[i + 1 - D0]);
     }
 }
 
@@ -229,12 +241,12 @@ __device__ __forceinline__ void pair_scatter(const KParams& kp, S* __restrict__ 
 template <typename T, bool EDGE>
 __device__ __forceinline__ float2 pair_ld_rest(const KParams& kp, const T* __restrict__ a,
                                                size_t extent, const PairNodes& pn) {
-    return pair_ld<T, EDGE>(kp, a, extent, pn, (size_t)0, 0, 0, 0);
+    return pair_ld<T, EDGE>(kp, a, extent, a, pn, 0u, 0, 0, 0);
 }
 template <typename T, bool EDGE>
 __device__ __forceinline__ void pair_st_rest(const KParams& kp, T* __restrict__ a, size_t extent,
                                              const PairNodes& pn, float2 v) {
-    pair_st<T, EDGE>(kp, a, extent, pn, (size_t)0, 0, 0, 0, v);
+    pair_st<T, EDGE>(kp, a, extent, a, pn, 0u, 0, 0, 0, v);
 }
 
 }  // namespace lbmgpu

@@ -397,6 +397,11 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
     if (k.storage != LBM_FP32 || k.scalar == LBM_SCALAR_Q27 || kp.wide ||
         (kp.flags & LBM_FLAG_ONE_NODE))
         return 0;
+    // Cumulant rows of up to 32 nodes step one node per thread (launch_cumulant_fp32),
+    // which a chain of half-empty pairs does not reach, us per step: 8x60x2500 241
+    // against 154, 20x60x1000 97 against 70, 32x60x75 8.0 against 7.2, 32x60x3125 305
+    // against 267 (65x60x307 62 against 72; BGK 32x60x625 48 against 51).
+    if (k.model == LBM_CUMULANT_Q27 && kp.nx <= 32) return 0;
     const int rows = (k.model == LBM_CUMULANT_Q27 ? 27 : 19) + (k.scalar == LBM_SCALAR_Q6 ? 6 : 7);
     const size_t plane_bytes = (size_t)kp.nxny * rows * sizeof(float);
     constexpr unsigned warps = CHAIN_WARPS;

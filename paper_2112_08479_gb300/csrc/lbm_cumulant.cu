@@ -396,10 +396,12 @@ cudaError_t launch_cumulant_chain(const KParams& kp, Kind k, bool odd, int nstep
 
 void fill_cumulant_sides(const KParams& kp, Sides& s) { pair_table(kp, 0, pair_view<13, 3>(s)); }
 
-// One node per thread in the arithmetic of the pairs: LBM_FLAG_ONE_NODE in FP32.
+// One node per thread in the arithmetic of the pairs: rows whose second half-segment
+// would stay idle (launch_cumulant_fp32) and LBM_FLAG_ONE_NODE in FP32.
 template <bool ODD, typename Off>
-__global__ void __launch_bounds__(128) cumulant_node_kernel(KParams kp, float* __restrict__ f,
-                                                            float* __restrict__ phi) {
+__global__ void __launch_bounds__(128, LBM_PAIR_MINB)
+    cumulant_node_kernel(KParams kp, float* __restrict__ f, float* __restrict__ phi) {
+    step_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= kp.nx) return;
     const Stencil st = make_stencil(kp, x, blockIdx.y, blockIdx.z);
@@ -416,14 +418,21 @@ template <bool WIDE>
 static cudaError_t launch_cumulant_fp32(const KParams& kp, bool odd, const Views& v,
                                         cudaStream_t st) {
     float *f = (float*)v.f, *phi = (float*)v.phi;
-    if (kp.flags & LBM_FLAG_ONE_NODE) {
+    const int ns = (kp.nx + 63) / 64, halves = (kp.nx + 31) / 32;
+    // Rows that end in the first half of their first or second segment leave a half or
+    // a quarter of the pairs' lanes idle, which costs more than one node per thread
+    // does.  One step of 6 M nodes, us, pairs / one node: nx = 8 1147 / 778, 32 361 /
+    // 265, 65 355 / 341, 96 282 / 275; not at 33 342 / 389, 64 243 / 260, 97 282 / 314,
+    // nor in the third segment, 130 316 / 323, 140 300 / 308.
+    if ((kp.flags & LBM_FLAG_ONE_NODE) || halves == 1 || halves == 3) {
         using Off = std::conditional_t<WIDE, size_t, unsigned>;
-        dim3 block(128), grid((kp.nx + 127) / 128, kp.ny, kp.nz);
-        if (odd) cumulant_node_kernel<true, Off><<<grid, block, 0, st>>>(kp, f, phi);
-        else cumulant_node_kernel<false, Off><<<grid, block, 0, st>>>(kp, f, phi);
+        const int w = pair_warps(halves);
+        dim3 block(32 * w), grid((halves + w - 1) / w, kp.ny, kp.nz);
+        if (odd) launch_after(cumulant_node_kernel<true, Off>, grid, block, st, kp, f, phi);
+        else launch_after(cumulant_node_kernel<false, Off>, grid, block, st, kp, f, phi);
         return cudaGetLastError();
     }
-    const int ns = (kp.nx + 63) / 64, w = pair_warps(ns);
+    const int w = pair_warps(ns);
     dim3 block(32 * w), grid((ns + w - 1) / w, kp.ny, kp.nz);
     launch_after(cumulant_pair_kernel<WIDE>, grid, block, st, kp, pair_view<13, 3>(*v.sides), f, phi,
                  odd);

@@ -53,7 +53,7 @@ def _check(p, steps, lead=0):
 
 @pytest.mark.parametrize("flags", [0, PX, PZ, PX | PZ])
 @pytest.mark.parametrize("kind", KINDS)
-@pytest.mark.parametrize("shape", [(64, 66, 66), (333, 17, 60), (3, 3, 1500), (40, 1, 4300)])
+@pytest.mark.parametrize("shape", [(64, 66, 66), (333, 17, 60), (35, 3, 1500), (40, 1, 4300)])
 def test_one_slot(shape, kind, flags):
     p = _params(shape, kind, flags)
     pl = _plan(p, 25)

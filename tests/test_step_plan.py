@@ -95,7 +95,7 @@ def _check_order(shape, steps, flags, model, sms=SMS):
     ((64, 66, 66), 24, 0, dict(slots=1, slabs=1, sweeps=24)),
     ((64, 66, 66), 25, PX | PZ, dict(slots=1, slabs=1, sweeps=25)),
     ((333, 17, 60), 24, PZ, dict(slots=1, slabs=1)),
-    ((3, 3, 1500), 24, PX, dict(slots=1, tiles=1)),
+    ((35, 3, 1500), 24, PX, dict(slots=1, tiles=1)),
     ((40, 1, 4300), 24, PZ, dict(slots=1, tiles=1)),
     # a wave over whole rows; one tile per plane; few planes
     ((300, 12, 600), 9, PX, dict(slots=4, slabs=1, sweeps=2)),
@@ -127,6 +127,9 @@ def test_which_calls_share_a_launch():
     assert _plan((256, 32, 64), 24)["steps"] == 24
     assert _plan((128, 8, 16), 1000)["steps"] == 0                  # too few rows
     assert _plan((1024, 64, 128), 100, PZ)["steps"] == 0            # no end for a wave
+    assert _plan((32, 60, 625), 100, 0, CUM)["steps"] == 0          # half-empty pairs
+    assert _plan((33, 60, 625), 100, 0, CUM)["steps"] == 100
+    assert _plan((32, 60, 625), 100)["steps"] == 100
     big = (1024, 64, 64)
     for kw in (dict(storage=lbm.LBM_FP16S), dict(storage=lbm.LBM_BF16S),
                dict(flags=lbm.LBM_FLAG_ONE_NODE), dict(model=CUM, scalar=lbm.LBM_SCALAR_Q27)):

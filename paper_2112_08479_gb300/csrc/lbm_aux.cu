@@ -194,6 +194,9 @@ __global__ void set_state_kernel(KParams kp, S* __restrict__ f, S* __restrict__ 
 // pass at even / odd parity, 25 / 37 with four; 256x32x64 with the D3Q27 scalar
 // 215 / 84, 27 / 29); a large one is bound by reading the state (2048x128x256
 // FP32 BGK 1109 / 1106 us, 1012 / 1049 with four; FP16 968 / 1015, 741 / 989).
+// Short spans under many columns keep one thread (launch_diag_columns), with its
+// registers bounded: the blocks of the odd gather came out at 92 (BGK) and 108
+// (cumulant) instead of 64 and 80, 57 against 47 us at 2048x1x512.
 // The loop over y stays rolled: as the compiler unrolled it, FP16 2048x128x256
 // with four threads took 1683 us at even parity, with two 1894.
 __device__ __forceinline__ unsigned fkey(float v) {
@@ -216,7 +219,7 @@ __device__ __forceinline__ void pair_add(float& s, float& c, float t, float d) {
 constexpr int DIAG_BX = 128;
 
 template <int Q, int SL, bool ODD, typename S, int DIAG_G>
-__global__ void __launch_bounds__(DIAG_BX * DIAG_G, Q == 19 ? 2 : 1) diag_columns_kernel(
+__global__ void __launch_bounds__(DIAG_BX * DIAG_G, DIAG_G == 1 ? (Q == 19 ? 8 : (SL == 27 ? 5 : 6)) : (Q == 19 ? 2 : 1)) diag_columns_kernel(
     KParams kp, const S* __restrict__ f, const S* __restrict__ phi, float* __restrict__ chibar,
     unsigned* __restrict__ colmax, double* __restrict__ part, float* __restrict__ fwpart,
     int* __restrict__ flags) {
@@ -698,13 +701,31 @@ static void launch_diag_columns(const KParams& kp, bool odd, const Views& v, cud
         kernel<<<grid, DIAG_BX * group, 0, st>>>(kp, (const S*)v.f, (const S*)v.phi, v.chibar,
                                                  v.colmax, v.part, v.fwpart, v.devflags);
     };
-    // the odd gather of the 27-velocity fluid prefers fewer rows at a time once the
-    // columns alone fill the chip (2048x128x256 FP32 / FP16: four 1542 / 1418 us, two
-    // 1491 / 1313; 1024x128x128, half of the limit: 402 / 373 and 404 / 363)
-    const bool many = (size_t)kp.nx * kp.nz >= (size_t)1 << 18;
-    if (!odd) run(diag_columns_kernel<Q, SL, false, S, 4>, 4);
-    else if (Q == 27 && many) run(diag_columns_kernel<Q, SL, true, S, Q == 27 ? 2 : 4>, 2);
-    else run(diag_columns_kernel<Q, SL, true, S, 4>, 4);
+    // Up to 2^14 columns leave warps to spare: four threads.  With more, one thread per
+    // column on spans below `least`, where the other threads of a group find no node or
+    // one and the block costs more than its loads; beyond, four, two for the odd gather
+    // of the 27-velocity fluid (fewer rows at a time).  2048 x 512 columns, us, one /
+    // two / four: FP32 BGK even ny = 1 47 / 66 / 90, 12 214 / 209 / 212, 16 279 / 270 /
+    // 268; odd 1 47 / 91 / 90, 16 284 / 333 / 309, 24 426 / 477 / 436; FP16 odd 24 369 /
+    // 436 / 419; cumulant even 4 97 / 96 / 120, 8 187 / 180 / 179; odd 4 117 / 144 / 225,
+    // 16 399 / 412 / 526, 32 770 / 773 / 910; D3Q27 scalar even 12 434 / 422 / 469, odd 8
+    // 315 / 301 / 390.
+    constexpr bool s16 = !std::is_same<S, float>::value;
+    constexpr int ODD_G = Q == 27 ? 2 : 4;
+    const int least = odd ? (Q == 19 ? (s16 ? 48 : 24) : (SL == 27 ? 8 : 24))
+                          : (SL == 27 ? 24 : (Q == 27 && !s16 ? 8 : 16));
+    const bool few = (size_t)kp.nx * kp.nz <= (size_t)1 << 14;
+    const bool one = !few && kp.ny < least;
+    if (one) {
+        if (odd) run(diag_columns_kernel<Q, SL, true, S, 1>, 1);
+        else run(diag_columns_kernel<Q, SL, false, S, 1>, 1);
+    } else if (!odd) {
+        run(diag_columns_kernel<Q, SL, false, S, 4>, 4);
+    } else if (few) {
+        run(diag_columns_kernel<Q, SL, true, S, 4>, 4);
+    } else {
+        run(diag_columns_kernel<Q, SL, true, S, ODD_G>, ODD_G);
+    }
 }
 
 cudaError_t launch_diag(const KParams& kp, Kind k, bool odd, const Views& v, double threshold,

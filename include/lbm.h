@@ -3,8 +3,8 @@
  *
  * The library advances the coupled fluid / scalar lattice Boltzmann model of
  * Adekanye et al., "GPU accelerated LBM simulations of dilute gravity
- * currents" (arXiv 2112.08479), one fused stream + collide kernel per time
- * step, on one CUDA device:
+ * currents" (arXiv 2112.08479) in fused stream + collide passes, on one CUDA
+ * device (a launch holds one time step, or several of one lbm_step call):
  *
  *   fluid   D3Q19 BGK with a Smagorinsky eddy viscosity and Guo forcing
  *           (Sec. 2.3.1, Eq. 17-26, 32-34), or D3Q27 cumulant
@@ -283,7 +283,8 @@ LBM_API lbm_status lbm_set_state(lbm_ctx* ctx, const float* src, int64_t step);
  *   lam_n = (dT/ds_n)^T lam_next + w_fw * dF_w(s_n)/ds_n,
  *   *dJdCs_dev += lam_next . dT/dC_s (s_n)   (BGK; the cumulant model has
  *                                            no C_s and adds nothing),
- * where T is the time step of lbm_step, s_n = state_n (canonical layout,
+ * where T is the time step as lbm_step_save takes it (lbm_step's up to FP32
+ * rounding), s_n = state_n (canonical layout,
  * device, (Q + NS) * N floats) is the state it was applied to, and lam_next,
  * lam_n are adjoint states in the canonical layout (device, (Q + NS) * N
  * floats; lam_next == NULL means zero).  lam_n must not alias lam_next or

@@ -17,12 +17,13 @@
 //
 // FP32: two nodes per thread, x and x + 32 of a 64-node segment of a row
 // (lbm_pair.cuh), collided in packed arithmetic.  Large boxes are bound by HBM
-// (208 bytes per node update, about 2 flop per byte): 32.6 G node updates/s at
-// 2048x128x256, 1.00 of the measured copy rate, as the form before it (pairs
-// of adjacent nodes, collided one after the other).  Boxes that fit the L2 and
-// rows of odd length were bound by instruction issue: 322 instructions per
-// node on both parities (456 / 634 before on even / odd steps) take the step
-// from 17.4 to 12.8 us at 256x32x64 and from 35.3 to 28.8 us at 333x47x59.
+// (208 bytes per node update, about 2 flop per byte) when steps are launched one
+// by one: 32.8 G node updates/s at 2048x128x256, 1.00 of the measured copy rate, as
+// the form before it (pairs of adjacent nodes, collided one after the other).
+// Boxes that fit the L2 and rows of odd length were bound by instruction issue: 322
+// instructions per node on both parities (456 / 634 before on even / odd steps)
+// took the step from 17.4 to 12.8 us at 256x32x64 and from 35.3 to 28.8 us at
+// 333x47x59, overlapped launches (launch_after) to 10.9 and 25.9.
 //
 // 16-bit storage: adjacent pairs (lbm_aa2.cuh) and, on even steps with nx a
 // multiple of 4, packed quads (lbm_quad.cuh); nx odd: one node per thread.

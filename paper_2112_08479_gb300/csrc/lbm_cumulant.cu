@@ -16,6 +16,11 @@
 
 namespace lbmgpu {
 
+// Below, up to the pair kernel, the one-node kernels in the contracted arithmetic.
+// FP32 steps of lbm_step with the D3Q7 scalar ran on them once, and the FP32 figures
+// of the D3Q7 instantiation date from then; they now serve, in FP32, saved steps and
+// objective trajectories, and the 16-bit storages and the D3Q27 scalar throughout.
+//
 // Minimum resident blocks per SM for the register allocator: the D3Q27 FCM
 // scalar holds more live values, so its instantiation gets its own setting,
 // per parity: odd steps 3 (168 registers, 36 bytes of spills; with 32-bit

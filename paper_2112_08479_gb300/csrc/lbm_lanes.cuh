@@ -51,7 +51,8 @@ struct Two {
 // 1 / a and sqrt(a): the hardware estimate (relative error about 1e-7) and one
 // Newton-Raphson step, to about half a unit in the last place, in packed
 // arithmetic.  sqrt takes a >= 0; the estimate is taken of at least 1e-37 so
-// that sqrt(0) = 0.
+// that sqrt(0) = 0.  (1 / a of a > 2^126 is 0, the hardware estimate's.  sqrt of
+// infinity is NaN, where the BGK collision would form inf / inf from infinity.)
 template <typename L>
 __device__ __forceinline__ typename L::V lane_rcp(typename L::V a) {
     const typename L::V r = L::rcp0(a);

@@ -47,10 +47,13 @@ def bytes_per_node(model="bgk", storage="fp32", scalar="q7") -> int:
         return (q + ns) * 2 * 4
     return (q + ns) * 2 * 2 + (4 if scalar != "q6" else 0)
 PROFILE = os.path.join(ROOT, "profiles", "aa_step_bgk_fp32_traffic.md")
-# the sources that define the headline step kernel (bgk_chain_kernel)
-KERNEL_SOURCES = ["paper_2112_08479_gb300/csrc/lbm_bgk.cu",
+# the sources that define the headline step kernel (bgk_chain_kernel) and the plan
+# of its launches, which decides its traffic
+KERNEL_SOURCES = ["paper_2112_08479_gb300/csrc/lbm_aux.cu",
+                  "paper_2112_08479_gb300/csrc/lbm_bgk.cu",
                   "paper_2112_08479_gb300/csrc/lbm_bgk_collide.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_chain.cuh",
+                  "paper_2112_08479_gb300/csrc/lbm_internal.h",
                   "paper_2112_08479_gb300/csrc/lbm_lanes.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_pair.cuh",
                   "paper_2112_08479_gb300/csrc/lbm_common.cuh"]
@@ -65,10 +68,10 @@ def kernel_hash() -> str:
 
 
 def profiled_traffic(nodes: int):
-    """DRAM bytes (read + write) per launch of the step kernel from the
-    committed ncu summary: the mean over the captured even and odd launches
-    when they ran on a box of `nodes` nodes, else the per-node figure scaled
-    to `nodes`.  (None, why) when the kernel changed since the capture."""
+    """DRAM bytes (read + write) per time step from the committed ncu summary:
+    of the captured launch divided by its steps when it ran on a box of `nodes`
+    nodes, else the per-node figure scaled to `nodes`.  (None, why) when the
+    kernel changed since the capture."""
     try:
         txt = open(PROFILE).read()
     except OSError:
@@ -76,10 +79,10 @@ def profiled_traffic(nodes: int):
     m = re.search(r"kernel_source_hash:\s*([0-9a-f]+)", txt)
     if not m or m.group(1) != kernel_hash():
         return None, "kernel changed since the capture"
-    full = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+-]+)", txt)
+    full = re.search(r"dram_bytes_per_(?:step|launch):\s*([0-9.eE+-]+)", txt)
     box = re.search(r"box_nodes:\s*([0-9]+)", txt)
     if full and box and int(box.group(1)) == nodes:
-        return float(full.group(1)), "ncu capture of this box (one even and one odd launch)"
+        return float(full.group(1)), "ncu capture of this box (per step of the captured launches)"
     b = re.search(r"dram_bytes_per_node_update:\s*([0-9.eE+-]+)", txt)
     if not b:
         return None, "no per-node figure"
@@ -348,6 +351,16 @@ def make_lattice(model="bgk", storage="fp32", scalar="q7", flags=0, **over):
     return lbm.Lattice(p, device="cuda")
 
 
+def step_launches(p, sms, n):
+    """Step kernels that lbm_step launches for n steps of a whole box p (lbm_params)
+    on a device of sms SMs: launches of several steps, then one per step left."""
+    from paper_2112_08479_gb300 import lbm
+    k = 0
+    while n and (together := lbm.lbm_step_plan(p, sms, n)["steps"]):
+        k, n = k + 1, n - together
+    return k + n
+
+
 def timed_loop(lat, steps, warmup, torch, inner=INNER, with_diag=True, kernel_events=True):
     """Returns (total seconds, mean step-kernel seconds, launches)."""
     s = lat.stream
@@ -371,12 +384,12 @@ def timed_loop(lat, steps, warmup, torch, inner=INNER, with_diag=True, kernel_ev
     torch.cuda.synchronize()
     total = t0.elapsed_time(t1) / 1e3
     kern = sum(a.elapsed_time(b) for a, b in evs) / 1e3 / (steps * inner)
-    # FP32 steps of one call share a launch (a whole box; slabs step one by one),
-    # except with the D3Q27 scalar: whole sweeps of three steps on the bench box,
-    # the rest one by one
-    chained = (getattr(lat, "peer", None) is None and lat.params.storage == 0
-               and lat.params.scalar != 2)
-    launches = steps * ((1 + inner % 3 if chained else inner) + (2 if with_diag else 0))
+    # (slabs step one by one)
+    per_call = inner
+    if getattr(lat, "peer", None) is None:
+        sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+        per_call = step_launches(lat.params.c(), sms, inner)
+    launches = steps * (per_call + (2 if with_diag else 0))
     return total, kern, launches
 
 
@@ -531,19 +544,24 @@ def run_ours(args, ws, rank, local):
     achieved = bpn * N / kern / 1e9
     headline = ((args.model, args.storage, args.scalar) == ("bgk", "fp32", "q7")
                 and args.workload == "config3")
+    shared = args.storage == "fp32" and args.scalar != "q27" and not slabs   # several steps a launch
     if args.storage == "fp32":
-        kname = "cumulant_step_kernel" if args.scalar == "q27" else f"{args.model}_chain_kernel"
+        kname = ("cumulant_step_kernel" if args.scalar == "q27"
+                 else f"{args.model}_{'chain' if shared else 'pair'}_kernel")
     else:
         kname = "bgk_step2_kernel" if args.model == "bgk" else "cumulant_step_kernel"
         if args.scalar == "q7" and WORKLOAD["nx"] % 4 == 0:
             kname = f"{args.model}_even4_kernel + {kname}"
     traffic, tsrc = profiled_traffic(N) if headline else (None, "not captured for this variant")
-    roof = {"bound": "hbm",
+    # a launch of several steps passes its state through HBM once per sweep of steps, so
+    # frac (state bytes of every step over the copy rate) may exceed 1 and HBM is not
+    # its bound; frac_dram has the bytes that ncu counted
+    roof = {"bound": "latency and issue" if shared else "hbm",
             "kernel": f"{kname} (AA even/odd, {args.storage.upper()})",
             "achieved": achieved, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
             "frac": achieved / peak, "traffic": traffic, "traffic_source": tsrc,
-            "algorithmic_bytes_per_launch": bpn * N, "mean_launch_ms": kern * 1e3,
-            # the same launch time against the DRAM bytes ncu counted, and the
+            "algorithmic_bytes_per_step": bpn * N, "mean_step_ms": kern * 1e3,
+            # the same step time against the DRAM bytes ncu counted, and the
             # algorithmic rate against the nominal 8 TB/s of the part
             "achieved_dram": traffic / kern / 1e9 if traffic else None,
             "frac_dram": traffic / kern / 1e9 / peak if traffic else None,

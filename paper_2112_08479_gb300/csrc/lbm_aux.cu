@@ -395,18 +395,36 @@ __global__ void adjoint_chi0_kernel(unsigned N, int Q, const float* __restrict__
     grad[n] = g;
 }
 
-// Rules of the chain (lbm_chain.cuh).
-int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, ChainPlan& out) {
+// Rules of the chain (lbm_chain.cuh).  State bytes of a plane:
+static double chain_plane_bytes(const KParams& kp, Kind k) {
+    const int rows = (k.model == LBM_CUMULANT_Q27 ? 27 : 19) + (k.scalar == LBM_SCALAR_Q6 ? 6 : 7);
+    return (double)kp.nxny * rows * sizeof(float);
+}
+
+// Whether the kind of box and the number of steps come into question; looked at
+// before the device is asked for its SMs, so that other calls do not pay for that.
+static bool chain_wanted(const KParams& kp, Kind k, int nsteps) {
     if (k.storage != LBM_FP32 || k.scalar == LBM_SCALAR_Q27 || kp.wide ||
         (kp.flags & LBM_FLAG_ONE_NODE))
-        return 0;
+        return false;
     // Cumulant rows of up to 32 nodes step one node per thread (launch_cumulant_fp32),
     // which a chain of half-empty pairs does not reach, us per step: 8x60x2500 241
     // against 154, 20x60x1000 97 against 70, 32x60x75 8.0 against 7.2, 32x60x3125 305
     // against 267 (65x60x307 62 against 72; BGK 32x60x625 48 against 51).
-    if (k.model == LBM_CUMULANT_Q27 && kp.nx <= 32) return 0;
-    const int rows = (k.model == LBM_CUMULANT_Q27 ? 27 : 19) + (k.scalar == LBM_SCALAR_Q6 ? 6 : 7);
-    const size_t plane_bytes = (size_t)kp.nxny * rows * sizeof(float);
+    if (k.model == LBM_CUMULANT_Q27 && kp.nx <= 32) return false;
+    // Steps that pay for the reset of the counters, the launch and the ramp (14 us on
+    // a box that fits L2), against one overlapped launch per step (launch_after), us
+    // per step: BGK 256x32x64 (55 MB) 16 steps 11.06, 24 10.87, 50 10.54 against
+    // 11.07; cumulant 256x32x64 (71 MB) 16 steps 15.40, 24 14.83 against 14.81;
+    // BGK 333x47x59 (96 MB) 8 steps 26.45, 12 25.14 against 26.00; 512x64x32 (109
+    // MB) 2 steps 31.0 against 31.9; 1024x64x128 2 steps 202 against 253.
+    const double state = chain_plane_bytes(kp, k) * kp.nz;
+    return nsteps >= (state < 80e6 ? 24 : (state < 105e6 ? 12 : 2));
+}
+
+int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, ChainPlan& out) {
+    if (!chain_wanted(kp, k, nsteps)) return 0;
+    const double plane_bytes = chain_plane_bytes(kp, k);
     constexpr unsigned warps = CHAIN_WARPS;
     // A box whose state stays in L2 needs no wave: steps in turn, one slot.
     constexpr double RESIDENT = 70e6;
@@ -424,15 +442,7 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
     // 2, 2.5, 3 measured 262, 210, 199, 198 us at 1024x64x128.
     constexpr double SLACK = 2.5;
     ChainParams& p = out.p;
-    const bool resident = plane_bytes * (double)kp.nz <= RESIDENT;
-    // Steps that pay for the reset of the counters, the launch and the ramp (14 us on
-    // a box that fits L2), against one overlapped launch per step (launch_after), us
-    // per step: BGK 256x32x64 (55 MB) 16 steps 11.06, 24 10.87, 50 10.54 against
-    // 11.07; cumulant 256x32x64 (71 MB) 16 steps 15.40, 24 14.83 against 14.81;
-    // BGK 333x47x59 (96 MB) 8 steps 26.45, 12 25.14 against 26.00; 512x64x32 (109
-    // MB) 2 steps 31.0 against 31.9; 1024x64x128 2 steps 202 against 253.
-    const double state = plane_bytes * (double)kp.nz;
-    if (nsteps < (state < 80e6 ? 24 : (state < 105e6 ? 12 : 2))) return 0;
+    const bool resident = plane_bytes * kp.nz <= RESIDENT;
     if (!resident && (kp.flags & LBM_FLAG_PERIODIC_Z)) return 0;   // a wave needs an end
     const unsigned nx = (unsigned)kp.nx, ny = (unsigned)kp.ny, nz = (unsigned)kp.nz;
     p.sync = nullptr;
@@ -466,10 +476,9 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
     if (CHAIN_COUNTERS + (size_t)P > kp.N) return 0;
     // whole sweeps of T steps; the rest is another call's (a sweep with idle slots
     // costs a whole one: cumulant 1024x64x128 with three slots, 4 steps 1415 us, 3
-    // steps and one 1166)
-    // ... and no more than keep every unit of the launch below 2^31, the range of Div
-    // and of a block's unit counter should one block take all of them: 1,820 steps of
-    // 2048x128x256.  The rest is the next launch's.
+    // steps and one 1166), and no more than keep every unit of the launch below 2^31,
+    // the range of Div and of a block's unit counter should one block take all of them:
+    // 1,820 steps of 2048x128x256.  The rest is the next launch's.
     const double tickets = 2147483648.0 / p.U - 1.0;
     const double sweeps = floor((tickets / ((double)T * bpt) - (double)(T - 1) * p.lag) / P / nslab);
     if (sweeps < 1.0) return 0;
@@ -496,6 +505,7 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
 cudaError_t chain_prepare(const KParams& kp, Kind k, const Views& v, int nsteps, bool odd,
                           ChainPlan& out, int& done, cudaStream_t st) {
     done = 0;
+    if (!chain_wanted(kp, k, nsteps)) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

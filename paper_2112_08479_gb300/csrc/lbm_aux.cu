@@ -411,7 +411,10 @@ static bool chain_wanted(const KParams& kp, Kind k, int nsteps) {
     // which a chain of half-empty pairs does not reach, us per step: 8x60x2500 241
     // against 154, 20x60x1000 97 against 70, 32x60x75 8.0 against 7.2, 32x60x3125 305
     // against 267 (65x60x307 62 against 72; BGK 32x60x625 48 against 51).
-    if (k.model == LBM_CUMULANT_Q27 && kp.nx <= 32) return false;
+    // BGK rows of one or two nodes leave nearly all of a unit empty: 1x60x80 9.6 against
+    // 7.3, 1x1000x600 1039 against 621, 2x60x5000 477 against 311 (4x60x80 7.1 against
+    // 7.3, 8x60x80 6.4 against 7.3).
+    if (kp.nx <= (k.model == LBM_CUMULANT_Q27 ? 32 : 2)) return false;
     // Steps that pay for the reset of the counters, the launch and the ramp (14 us on
     // a box that fits L2), against one overlapped launch per step (launch_after), us
     // per step: BGK 256x32x64 (55 MB) 16 steps 11.06, 24 10.87, 50 10.54 against

@@ -130,6 +130,8 @@ def test_which_calls_share_a_launch():
     assert _plan((32, 60, 625), 100, 0, CUM)["steps"] == 0          # half-empty pairs
     assert _plan((33, 60, 625), 100, 0, CUM)["steps"] == 100
     assert _plan((32, 60, 625), 100)["steps"] == 100
+    assert _plan((2, 60, 5000), 100)["steps"] == 0                  # nearly empty units
+    assert _plan((3, 60, 5000), 100)["steps"] == 100
     big = (1024, 64, 64)
     for kw in (dict(storage=lbm.LBM_FP16S), dict(storage=lbm.LBM_BF16S),
                dict(flags=lbm.LBM_FLAG_ONE_NODE), dict(model=CUM, scalar=lbm.LBM_SCALAR_Q27)):

@@ -108,8 +108,8 @@ typedef enum lbm_storage {
 #define LBM_FLAG_TEST_STALL 32 /* test hook of the failure path of kernels with bounded waits.
                                   With LBM_FLAG_TMA_STAGED each block's first tile is
                                   announced on its barrier but never copied; in a launch of
-                                  several steps (lbm_step_plan) the first finished item is
-                                  not counted.  The waits for these cannot end; every wait
+                                  several steps (lbm_step_plan) the first tile's count of
+                                  finished items starts one short.  The waits for these cannot end; every wait
                                   gives up after 0.1 s, the kernel sets LBM_DEVFLAG_TIMEOUT
                                   and returns (lbm_diag then reports LBM_ERR_TIMEOUT); no
                                   fault, no hang */

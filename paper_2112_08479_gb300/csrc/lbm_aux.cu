@@ -499,8 +499,7 @@ int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, Ch
     p.nslab.set(nslab);
     p.sw.set(sw);
     p.Ud.set(p.U);
-    p.stall = (kp.flags & LBM_FLAG_TEST_STALL) != 0;
-    p.limit_ns = p.stall ? CHAIN_STALL_NS : CHAIN_LIMIT_NS;
+    p.limit_ns = (kp.flags & LBM_FLAG_TEST_STALL) ? CHAIN_STALL_NS : CHAIN_LIMIT_NS;
     out.grid = sms < p.total ? sms : p.total;
     return nsteps;
 }
@@ -516,7 +515,10 @@ cudaError_t chain_prepare(const KParams& kp, Kind k, const Views& v, int nsteps,
     done = chain_plan(kp, k, (unsigned)sms, nsteps, odd, out);
     if (!done) return cudaSuccess;
     out.p.sync = reinterpret_cast<unsigned*>(v.stage);
-    return cudaMemsetAsync(out.p.sync, 0, (CHAIN_COUNTERS + (size_t)out.p.P.d) * sizeof(unsigned), st);
+    e = cudaMemsetAsync(out.p.sync, 0, (CHAIN_COUNTERS + (size_t)out.p.P.d) * sizeof(unsigned), st);
+    if (e == cudaSuccess && (kp.flags & LBM_FLAG_TEST_STALL))
+        e = cudaMemsetAsync(out.p.sync + CHAIN_COUNTERS, 0xff, sizeof(unsigned), st);
+    return e;
 }
 
 // ---------------------------------------------------------------------------

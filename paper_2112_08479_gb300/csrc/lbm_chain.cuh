@@ -78,7 +78,6 @@ struct ChainParams {
     Div sw;             // warp segments per row and slab
     Div Ud;             // U
     unsigned long long limit_ns;   // longest wait for a counter
-    int stall;          // LBM_FLAG_TEST_STALL: the first item of the first tile is not counted
 };
 
 constexpr unsigned long long CHAIN_LIMIT_NS = 10000000000ull;   // only a defect waits that long
@@ -287,8 +286,7 @@ __device__ __forceinline__ void chain_run(const KParams& kp, const ChainParams& 
                 const ChainItem im = sh.item[lane];
                 fence_gpu();
                 if (full) {
-                    const bool held = cp.stall && (im.nu | im.z | im.tile | im.b) == 0;
-                    if (!held) red_add(done + ((unsigned)im.z * cp.M.d + (unsigned)im.tile), 1u);
+                    red_add(done + ((unsigned)im.z * cp.M.d + (unsigned)im.tile), 1u);
                     sh.finished[lane] = 0;
                     ++seen;
                     sts_release(&sh.freed[lane], seen);
@@ -318,7 +316,8 @@ struct ChainPlan {
 int chain_plan(const KParams& kp, Kind k, unsigned sms, int nsteps, bool odd, ChainPlan& out);
 
 // The plan on the current device, with its counters in the staging buffer of
-// lbm_set_scalar (whose contents are not kept between calls), zeroed on the stream.
+// lbm_set_scalar (whose contents are not kept between calls), zeroed on the stream
+// (LBM_FLAG_TEST_STALL: the first tile's starts one short, and is never full).
 cudaError_t chain_prepare(const KParams& kp, Kind k, const Views& v, int nsteps, bool odd,
                           ChainPlan& out, int& done, cudaStream_t st);
 

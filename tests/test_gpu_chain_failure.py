@@ -1,6 +1,6 @@
-"""Failure path of a launch of several steps: LBM_FLAG_TEST_STALL leaves one
-finished item uncounted (a flag that nothing sets) and sets the limit of the waits
-to 0.1 s.  The waits for it run out, every block ends, LBM_DEVFLAG_TIMEOUT is set,
+"""Failure path of a launch of several steps: LBM_FLAG_TEST_STALL starts one
+tile's count of finished items one short (a flag that nothing sets) and sets the
+limit of the waits to 0.1 s.  The waits for it run out, every block ends, LBM_DEVFLAG_TIMEOUT is set,
 lbm_diag reports LBM_ERR_TIMEOUT and the device stays usable.  No fault, no trap,
 no hang is provoked."""
 import ctypes
